@@ -84,6 +84,23 @@ size_t smem_of(const labs_instance* h, int64_t n) {
     return s;
 }
 
+// Warps per CTA that a mapping's wpb becomes for these instances (cta_warps
+// of the largest population, whose footprint every warp of the launch gets).
+int cta_warps_of(const labs_instance* h, int64_t n, int wpb, int wps) {
+    const labs_instance* top = nullptr;
+    size_t most = 0;
+    for (int64_t i = 0; i < n; ++i) {
+        const size_t b = lgpu::mts_smem_per_warp(h[i].N, h[i].K);
+        if (b > most) {
+            most = b;
+            top = h + i;
+        }
+    }
+    if (top == nullptr) return wpb;
+    const int nw = 2 * ((top->N + 63) / 64);
+    return lgpu::cta_warps(wpb, wps, static_cast<size_t>(top->K) * (nw + 1) * 4, nw);
+}
+
 std::vector<int32_t> queue_order(const labs_instance* h, int64_t n, int order) {
     std::vector<int32_t> idx(static_cast<size_t>(n));
     std::iota(idx.begin(), idx.end(), 0);
@@ -221,8 +238,10 @@ int32_t labs_autotune(const labs_instance* h_inst, int64_t n, labs_stream_t stre
         for (int wpb : {1, 2, 4, 8}) {
             if (wpb < wps) continue;
             int maxb = 0;
-            if (e == cudaSuccess) e = lgpu::batch_prepare(nwmax, wps, wpb, spw, &maxb);
+            const int cta = cta_warps_of(h_inst, n, wpb, wps);
+            if (e == cudaSuccess) e = lgpu::batch_prepare(nwmax, wps, cta, spw, &maxb);
             if (e != cudaSuccess) break;
+            maxb /= wpb / cta;  // CTAs of wpb warps
             for (int bps : {1, 2, 4, 8, 16}) {
                 if (bps > maxb) break;
                 // more resident replicas than instances x 2 cannot help
@@ -230,7 +249,7 @@ int32_t labs_autotune(const labs_instance* h_inst, int64_t n, labs_stream_t stre
                 for (int rep = warmed ? 0 : 1; rep >= 0 && e == cudaSuccess; --rep) {
                     e = cudaMemsetAsync(d.queue, 0, sizeof(unsigned long long), s);
                     if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-                    if (e == cudaSuccess) e = lgpu::launch_batch(a, nwmax, wps, sms * bps, wpb, s);
+                    if (e == cudaSuccess) e = lgpu::launch_batch(a, nwmax, wps, sms * bps * (wpb / cta), cta, s);
                     if (e == cudaSuccess) e = cudaEventRecord(e1, s);
                     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                 }
@@ -285,19 +304,19 @@ int32_t labs_batch_create(const labs_instance* h_inst, int64_t n, const labs_map
     b->d_out = d.out;
     b->d_queue = d.queue;
     int maxb = 0;
-    if (e == cudaSuccess) e = lgpu::batch_prepare(b->nwmax, wps_of(m), m.warps_per_block, b->smem_per_warp, &maxb);
+    const int cta = cta_warps_of(h_inst, n, m.warps_per_block, wps_of(m));
+    if (e == cudaSuccess) e = lgpu::batch_prepare(b->nwmax, wps_of(m), cta, b->smem_per_warp, &maxb);
     if (e == cudaSuccess && maxb < 1) {
         labs_batch_destroy(b);
         return fail(LABS_EINVAL, "mapping does not fit on an SM (warps_per_block=%d)", m.warps_per_block);
     }
-    b->blocks = sm_count() * std::min(m.blocks_per_sm, std::max(maxb, 1));
+    b->blocks = sm_count() * std::min(m.blocks_per_sm * (m.warps_per_block / cta), std::max(maxb, 1));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t le = cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned long long), b->cap);
         if (le == cudaSuccess)
-            le = lgpu::launch_batch(args_of(d, n, b->smem_per_warp), b->nwmax, wps_of(m), b->blocks,
-                                    m.warps_per_block, b->cap);
+            le = lgpu::launch_batch(args_of(d, n, b->smem_per_warp), b->nwmax, wps_of(m), b->blocks, cta, b->cap);
         e = cudaStreamEndCapture(b->cap, &b->graph);
         if (le != cudaSuccess) e = le;
     }

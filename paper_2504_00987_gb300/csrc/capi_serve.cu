@@ -443,7 +443,9 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
         return nullptr;
     }
     const int top = class_of(o->max_N);
-    if (lgpu::serve_smem_per_warp(kClassNw[top], o->max_K) * o->warps_per_block > 227u * 1024u) {
+    const size_t pop_max = static_cast<size_t>(o->max_K) * (kClassNw[top] + 1) * 4;
+    const int cta = lgpu::cta_warps(o->warps_per_block, 1, pop_max, kClassNw[top]);
+    if (lgpu::serve_smem_per_warp(kClassNw[top], o->max_K) * cta > lgpu::kCtaSmem) {
         fail(LABS_EINVAL, "max_N/max_K populations of one block exceed shared memory");
         return nullptr;
     }
@@ -462,7 +464,8 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
         return nullptr;
     }
     s->opts = *o;
-    s->pair_wpb = std::max(2, o->warps_per_block);
+    s->opts.warps_per_block = cta;
+    s->pair_wpb = std::max(2, cta);
     cudaGetDevice(&s->device);
     // the arena: hbm_budget_bytes, or room for max_slots requests of (max_N, max_K)
     labs_request biggest{};
@@ -485,13 +488,13 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
     for (int c = 0; c <= top && e == cudaSuccess; ++c) {
         s->cls_smem[c] = lgpu::serve_smem_per_warp(kClassNw[c], o->max_K);
         int blocks = 0;
-        e = lgpu::serve_blocks_per_sm(kClassNw[c], 1, o->warps_per_block, s->cls_smem[c], &blocks);
+        e = lgpu::serve_blocks_per_sm(kClassNw[c], 1, cta, s->cls_smem[c], &blocks);
         if (e == cudaSuccess && blocks < 1) {
             fail(LABS_EINVAL, "the quantum kernel for %d-word sequences does not fit on an SM", kClassNw[c]);
             free_server(s);
             return nullptr;
         }
-        s->cls_cap[c] = static_cast<int64_t>(blocks) * o->warps_per_block * sm_count();
+        s->cls_cap[c] = static_cast<int64_t>(blocks) * cta * sm_count();
         if (e == cudaSuccess && o->warps_per_request == 2 && lgpu::serve_pairs_supported(kClassNw[c])) {
             int b2 = 0;
             e = lgpu::serve_blocks_per_sm(kClassNw[c], 2, s->pair_wpb, s->cls_smem[c], &b2);

@@ -12,6 +12,25 @@ namespace lgpu {
 
 constexpr int kWarpsPerBlock = 4;
 
+// Shared scratch of one warp's tabu search over nw 32-bit words: V and C (64 nw
+// ints each) and the spins (96 nw bytes); see tabu_search.
+constexpr size_t tabu_scratch_bytes(int nw) { return 608u * static_cast<size_t>(nw); }
+
+// Shared memory of one CTA.
+constexpr size_t kCtaSmem = 227u * 1024u;
+
+// A mapping or a server with wpb warps per CTA is accepted while wpb warps of
+// `pop` population bytes and 256 nw bytes fit a CTA.  The search's scratch is
+// larger: where wpb warps do not fit with it, the CTA runs half as many (or a
+// quarter), which no result depends on.  `least`: warps that belong together.
+inline int cta_warps(int wpb, int least, size_t pop, int nw) {
+    const auto padded = [](size_t b) { return (b + 15) & ~size_t{15}; };
+    const size_t links = least == 2 ? 128 : 0;  // static shared memory of the kernels on warp pairs
+    if (padded(pop + 256u * static_cast<size_t>(nw)) * wpb + links > kCtaSmem) return wpb;  // refused by the caller
+    while (wpb > least && padded(pop + tabu_scratch_bytes(nw)) * wpb + links > kCtaSmem) wpb /= 2;
+    return wpb;
+}
+
 struct MtsArgs {
     int32_t N, K;
     uint32_t p_comb_u32, p_mut_u32;

@@ -101,8 +101,7 @@ __device__ void serve_slot(const ServeArgs& a, int i, int slot, const labs_insta
             }
             if (over) break;
         }
-        // correlations updated per k (PERK): a request's warp mostly runs alone on its sub-partition
-        used += replica_generation<NW, false, false, WPS, HALF, true>(cfg, st, pop, popE, Cs, nullptr, 0,
+        used += replica_generation<NW, false, false, WPS, HALF>(cfg, st, pop, popE, Cs, nullptr, 0,
                                                                       trace_len, nullptr, lane, link, &xseq);
     }
     if (HALF != 0) return;
@@ -156,8 +155,8 @@ __global__ void __launch_bounds__(256, WPS == 2 ? 1 : 0) serve_quantum_kernel(co
 int serve_class_nw(int N) { return N <= 64 ? 2 : N <= 96 ? 3 : N <= 128 ? 4 : N <= 160 ? 5 : N <= 192 ? 6 : 8; }
 
 size_t serve_smem_per_warp(int nw, int K) {
-    // population (K x nw words), energies (K), two buffers of C_k (64 nw)
-    const size_t bytes = (static_cast<size_t>(K) * nw + static_cast<size_t>(K) + 64u * nw) * 4u;
+    // population (K x nw words), energies (K), the tabu search's scratch
+    const size_t bytes = (static_cast<size_t>(K) * nw + static_cast<size_t>(K)) * 4u + tabu_scratch_bytes(nw);
     return (bytes + 15) & ~static_cast<size_t>(15);
 }
 

@@ -12,18 +12,16 @@
 // where S_j = sum_m w_m [popc(t_m & X_j) + popc(t_m & Y_j)] over the
 // two's-complement planes t_m of C_k (from warp ballots), X_j = pivot >> j
 // (bit k = b_{j+k}) and Y_j the mirrored window (bit k = b_{j-k}); T_j comes
-// from prefix sums of C_k.  After every move R_j is updated exactly instead
-// of re-scored (the identity is derived above tabu_search), so a step costs
-// about one bit plane of the from-scratch scoring.  Arithmetic is exact int32.
+// from prefix sums of C_k.  After every move each neighbour's energy change
+// is updated exactly in O(1) from C_k and the self-convolution V_m of the
+// spins (the identity stands above tabu_search), so a step never goes back to
+// the bits.  Arithmetic is exact int32.
 //
-// Work split: lane l scores neighbours j = l + 32q and keeps their R_j and
-// tabu expiry in registers; C_k before and after the move sit in two
-// warp-private shared-memory buffers.  The admissible minimum is one
-// redux.sync.min over packed (E_j, j) keys, the ties are counted by one
-// redux.sync.add, and a tie pick by the step's draw in ascending j uses
-// ballots only when it is not the lowest minimiser.  Applying the move
-// flips the pivot, recomputes (short sequences) or updates C_k, updates
-// every R_j and sets the tenure.
+// Work split: lane l owns the neighbours j = l + 32q: their keys (energy
+// change, index and spin in one int), tabu expiry and spins in registers; V,
+// C and the spins also in the warp's slice of shared memory, where the move
+// shifts them against each other.  The admissible minimum is one
+// redux.sync.min over the keys; ballots resolve a tie only where there is one.
 #pragma once
 
 #include <climits>
@@ -295,44 +293,95 @@ __device__ __forceinline__ void pivot_windows(const uint32_t (&B)[NW], const uin
     }
 }
 
+// Scratch of one warp's tabu search (ints): V (2 NB), C (2 NB), spins (3 NB
+// bytes), NB = 32 NW; a multiple of 16 bytes.
+template <int NW>
+constexpr int kTabuScratchInts = 128 * NW + 24 * NW;
+
+// V_m = sum_a s_a s_{m-a} (terms outside 0..N-1 dropped) for m = lane + 32i,
+// i < 2 NW, from the bits of the sequence and its mirror image.
+template <int NW>
+__device__ __forceinline__ void store_self_convolution(const uint32_t (&B)[NW], const uint32_t (&RL)[NW], int N,
+                                                       int lane, int32_t* __restrict__ Vs) {
+    // Z[x + 1] = word x of RL >> (31 - lane), x = -1 .. NW-1: bit i of word
+    // w + NW - 1 - i' is b_{m-a} for m = lane + 32 i', a = 32 w + i
+    uint32_t Z[NW + 1];
+    Z[0] = __funnelshift_r(0u, RL[0], 31 - lane);
+#pragma unroll
+    for (int x = 0; x < NW; ++x) Z[x + 1] = __funnelshift_r(RL[x], x + 1 < NW ? RL[x + 1] : 0u, 31 - lane);
+#pragma unroll
+    for (int i = 0; i < 2 * NW; ++i) {
+        const int m = lane + 32 * i;
+        const int lo = max(0, m - N + 1), hi = min(m, N - 1);  // a in [lo, hi]
+        int diff = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const int x = w + NW - 1 - i;  // compile-time
+            if (x >= -1 && x < NW)
+                diff += __popc((B[w] ^ Z[x + 1]) & word_lowmask(w, hi + 1) & ~word_lowmask(w, lo));
+        }
+        Vs[m] = max(hi - lo + 1, 0) - 2 * diff;
+    }
+}
+
 // One tabu search from `seq` (warp-uniform).  On return `seq` holds
 // bestSeqTS.  Draws: step t uses Philox(instance, g, t, 4): x tie, y tenure.
 // FIX_FIRST: bit 0 (s_1) is never a candidate move.
-// `Cs` is warp-private shared scratch of 64*NW ints (two buffers of C_k).
+// `Cs` is warp-private shared scratch of kTabuScratchInts<NW> ints.
 // With TRACE, `trace` receives {g, t, j, E} per step while trace_len <
 // trace_cap.
 //
-// Neighbour scores are kept between steps.  With
-//   R_j = sum_k C_k (s~_{j+k} + s~_{j-k})     (s~_i = s_i inside 0..N-1, else 0)
-//   M_j = sum_{k>=1} s~_{j+k} s~_{j-k},
-// the energy after flipping j is E_j = E + 4(N-1) + 8 M_j - 4 s_j R_j (the
-// delta_k(j)(2 C_k + delta_k(j)) sum of Table I, expanded).  R_j is set up
-// once per search on the bit planes of C_k; after the move p (s_p before
-// it, C and C' the correlations before and after, d = |p - j|, s'_j after
-// the move) it changes exactly by
-//   R'_j = R_j - 2 s_p (C_d + C'_d + F_j) - 2 s'_j          (j != p)
-//   R'_p = R_p - 2 s_p (N - 1 + 2 M_p)
-// with F_j = sum_{k>=1} s~_{p+k} s~'_{j-k} + sum_{k>=1} s~_{p-k} s~'_{j+k}
-// (s~' after the move).  Derivation: R'_j - R_j = sum_k C_k (s~'-s~)
-// (terms j+-k = p: -2 s_p C_d) + sum_k delta_k(p) (s~'_{j+k} + s~'_{j-k});
-// the second sum pairs the windows of p and j: its same-direction pairs
-// (p+k, j+k), (p-k, j-k) cover every product of C'_d except s'_p s'_j, and
-// its crossed pairs are F_j.  At j = p the crossed pairs give F_p = 2 M_p and
-// s'_p = -s_p, so the first line gives the second when C_0 + C'_0 = N: the
-// two buffers hold ceil(N/2) and floor(N/2) at k = 0 and one update serves
-// every j.  F_j is two masked popcounts over the windows of p and j (the
-// crossed pairs agree or disagree), C_d and C'_d are read from the two
-// shared buffers, so a step costs about one bit plane of the from-scratch
-// scoring instead of one per bit of max |C_k|.
+// Every neighbour's energy change D_j = E_j - E is kept between steps, and a
+// step costs O(N) for the whole neighbourhood.  With s~_i = s_i inside
+// 0..N-1 (0 outside), C_k = sum_i s~_i s~_{i+k} and V_m = sum_a s~_a s~_{m-a},
+// the move p (s_p before it, sigma = s_p s_j) changes
+//   D'_j = D_j + 8 sigma (2 C_{|j-p|} + V_{p+j}) - 16 (s_p s~_{2j-p} + s_j s~_{2p-j}) - 32
+//   V'_{p+j} = V_{p+j} - 4 sigma,   C'_{|j-p|} = C_{|j-p|} - 2 sigma - 2 s_p s~_{2p-j}   (j != p)
+//   D'_p = -D_p,                    V'_{2p} = V_{2p}
+// (C and V on the right before the move; no other V_m or C_k changes).
+// Derivation: D_j = 4(N-1) + 8 M_j - 4 s_j R_j with M_j = sum_{k>=1}
+// s~_{j+k} s~_{j-k} and R_j = sum_k C_k (s~_{j+k} + s~_{j-k}).  M_j has one
+// product with s_p, at the mirror position 2j - p.  R'_j - R_j is -2 s_p C_d
+// (d = |j-p|, the two terms j +- k = p) plus sum_k delta_k(p) (s~'_{j+k} +
+// s~'_{j-k}) with delta_k(p) = -2 s_p (s~_{p+k} + s~_{p-k}), s~' after the
+// move: its pairs (p+-k, j+-k) of one direction make C'_d without the
+// product s'_p s'_j, and its crossed pairs (p+k, j-k) all have the index sum
+// p + j, so they make V_{p+j} but for the products of s_p and s_j.
+// With c' = C'_{|j-p|} the same change reads, in units of 4,
+//   D'_j / 4 = D_j / 4 + 2 s_p (s_j (C_{|j-p|} + c' + V_{p+j}) - 2 s~_{2j-p}) - 4,
+// six multiply-adds a neighbour with the updates of C and V.
 //
-// WPS = 2 (two warps per replica, HALF = which one): the warp scores and
-// updates only the neighbours j = lane + 32q of its half of q, keeps its own
-// copy of everything else (pivot, correlations, bestSeqTS), and the two
-// minima meet through `link`; the lower half's neighbours come first in
-// ascending j for the tie pick.  Both warps take every decision from the
-// same values, so they run the same steps; `xseq` counts the pair's
-// exchanges.  A bounded wait that runs out ends the search with fault set.
-template <int NW, bool TRACE, bool FIX_FIRST = false, int WPS = 1, int HALF = 0, bool PERK = false>
+// Lane l owns j = l + 32q: key K_j, tabu expiry and s_j in registers.  Keys
+// are D_j / 4 << 9 | j << 1 | (s_j == +1): D_j is a multiple of 4 below 2^23
+// in magnitude for N <= 256, one redux.sync.min gives the least change, its
+// lowest index and that spin.  In shared memory: V; C at both +d and -d, so
+// that C_{|j-p|} of consecutive lanes is consecutive words and needs no
+// absolute value; -2 s~ as bytes with NB zeros on either side.  Lanes with
+// j >= N hold s_j = 0 and a key that never changes.
+//
+// What bounds it: one warp's steps are a serial chain (test the keys, reduce,
+// load what the move shifts, update, next test).  On GB300 redux.sync.min
+// takes 18 cycles, a shared load 29, a multiply-add 5, a compare whose
+// predicate is used at once 14, a vote with a branch on it 37.  So the keys
+// are tested through selects and a minimum tree (predicated minima made a
+// chain that cost 70 cycles more at N = 64 and 250 at N = 120), and the move
+// of the lowest minimiser is scored before the vote on ties is looked at and
+// scored again in the rarer case that another one is drawn (36 cycles less at
+// N = 64, 72 at N = 120).  A ballot and a popcount per 32 neighbours in place
+// of that one vote took 14 cycles more at N = 64 and 37 at N = 120; keeping
+// the best sequence without a branch, 21 and 1 more.
+// Measured, cycles a step, one warp / two / four on an SM sub-partition:
+// N = 64 217 / 295 / 510, N = 120 343 / 453 / 758, N = 192 414 / 574 (two
+// popcounts of windows per neighbour and word, before: one launch of 1,024
+// replicas x 10^5 steps at N = 64 took 559 cycles a step).
+//
+// WPS = 2 (two warps per replica, HALF = which one): the warp keeps the keys
+// of its half of q and its own copy of V, C and the spins; the two minima
+// meet through `link`; the lower half's neighbours come first in ascending j
+// for the tie pick.  Both warps take every decision from the same values, so
+// they run the same steps; `xseq` counts the pair's exchanges.  A bounded
+// wait that runs out ends the search with fault set.
+template <int NW, bool TRACE, bool FIX_FIRST = false, int WPS = 1, int HALF = 0>
 __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key,
                                const uint32_t inst, const uint32_t g, const int max_iter,
                                const int64_t budget, int32_t* __restrict__ Cs,
@@ -342,65 +391,33 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     static_assert(WPS == 1 || (WPS == 2 && NW % 2 == 0 && HALF >= 0 && HALF < 2), "warps per sequence");
     constexpr int NB = 32 * NW;
     constexpr int QB = HALF * (NW / WPS), QE = (HALF + 1) * (NW / WPS);  // this warp's q
-    // Correlations after a move are recomputed from the pivot's windows when
-    // they are short (fewer ALU-pipe instructions than the per-k update: at
-    // N = 64 the per-k update measured 11-15 % slower with two warps per SM
-    // sub-partition) and updated per k otherwise.  PERK (the batch and
-    // service kernels, whose warps mostly run alone on their sub-partition,
-    // so that a step's dependency chain sets its time) always updates per k:
-    // the update needs only the move's windows, not the flipped pivot, which
-    // measured 13 % less time for the 512-instance uneven batch on GB300 and
-    // 8 % less median service latency.
-    constexpr bool kRecompute = NW <= 4 && !PERK;
-    uint32_t B[NW], RL[NW], Bb[NW];
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        B[w] = seq[w];
-        Bb[w] = seq[w];
-    }
-    reverse_bits<NW>(B, RL);
-    uint32_t XB[NW], YB[NW];
-    pivot_windows<NW>(B, RL, lane, XB, YB);
-    int32_t c[NW];
-    correlations<NW>(B, N, lane, c);
-    int32_t E;
+    // A drawn tie is scored by a second copy of the scoring code from three
+    // words on, and through the loop of the first where two words make that
+    // copy as long as the rest of the step (cycles a step, one warp alone:
+    // N = 64 232 with the copy, 217 without; N = 120 343 and 355; N = 192 414
+    // and 443).
+    constexpr bool kRecompute = NW <= 4 ? NW > 2 : true;
+    constexpr int32_t kLow = 511;  // key bits below the energy change
+    constexpr int32_t kNone = INT_MAX & ~kLow;  // no candidate: above every key, low bits those of j = 0
+    int32_t* const Vs = Cs;                                     // V_m, m = 0 .. 2 NB - 1
+    int32_t* const C0 = Cs + 3 * NB;                            // C_d at C0[d] and C0[-d]
+    int8_t* const S0 = reinterpret_cast<int8_t*>(Cs + 4 * NB) + NB;  // -2 s~_i, i = -NB .. 2 NB - 1
+    int32_t s[NW], c[NW];
+    correlations<NW>(seq, N, lane, c);
+    int32_t E_best;
     {
         int32_t sq = 0;
 #pragma unroll
         for (int q = 0; q < NW; ++q) sq += c[q] * c[q];
-        E = __reduce_add_sync(kFull, sq);
+        E_best = __reduce_add_sync(kFull, sq);
     }
-    int32_t E_best = E;
-    // Per-search constants of the lane's neighbours j = lane + 32q: validity,
-    // L_j = min(j, N-1-j) and the masks of k in [1, L_j] (M_j), the range
-    // masks of the forward windows (bits k <= N-1-j of X_j, word i = q + w),
-    // and for the recomputed correlations the masks of i < N - k.
-    int32_t tabu[NW], Lq[NW];
-    uint32_t mmask[NW][NW], mX[NW];
-    uint32_t jvalid = 0;  // bit q: j < N and j may move
-#pragma unroll
-    for (int q = 0; q < NW; ++q) mX[q] = word_lowmask(q, N - lane);
-#pragma unroll
-    for (int q = QB; q < QE; ++q) {
-        const int j = lane + 32 * q;
-        Lq[q] = min(j, N - 1 - j);
-        const bool movable = j < N && !(FIX_FIRST && j == 0);
-        jvalid |= (movable ? 1u : 0u) << q;
-        // A neighbour that may not move is already excluded by jvalid; for
-        // two-word sequences it also gets an expiry that never passes, which
-        // changes no result but measured 2.8 % less time per launch at N = 64
-        // on GB300 (code generation; the same line cost 0.4-5 % at N = 92..160).
-        tabu[q] = (NW == 2 && !movable) ? INT_MAX : 0;
-#pragma unroll
-        for (int w = 0; w <= q && w + q < NW; ++w)
-            mmask[q][w] = word_lowmask(w, Lq[q] + 1) & (w == 0 ? ~1u : kFull);
-    }
-    const uint32_t low_l = (lane == 31) ? kFull : ((2u << lane) - 1u);  // bits 0..lane
     // R_j = 2 S_j - T_j from the bit planes of C_k (S_j) and the prefix sums
     // of C_k (T_j = PC(j) + PC(N-1-j)), once per search.
-    int32_t R[NW];
+    int32_t K[NW], tabu[NW];
     {
-        uint32_t par[NW];
+        uint32_t RL[NW], XB[NW], YB[NW], par[NW];
+        reverse_bits<NW>(seq, RL);
+        pivot_windows<NW>(seq, RL, lane, XB, YB);
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
             const uint32_t alt = ((N - 32 * w) & 1) ? 0x55555555u : 0xAAAAAAAAu;  // (N - k) odd
@@ -418,232 +435,231 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
         score_dispatch<NW>(plane_count<NW>(c), c, par, X, Y, S);
         prefix_own<NW>(c, lane, pc);
         mirror_terms<NW>(pc, N, lane, Cs, T);
+        store_self_convolution<NW>(seq, RL, N, lane, Vs);
 #pragma unroll
-        for (int q = QB; q < QE; ++q) R[q] = 2 * S[q] - T[q];
-    }
-    // C_k of the pivot (Ccur) and after the move (Cnxt), k = 1 .. NB-1 (0 past
-    // N-1); slot k = 0 holds ceil(N/2) in one buffer and floor(N/2) in the
-    // other and is never rewritten (see the update of R_p above).
-    int32_t* Ccur = Cs;
-    int32_t* Cnxt = Cs + NB;
-#pragma unroll
-    for (int q = 0; q < NW; ++q) Ccur[lane + 32 * q] = c[q];
-    if (lane == 0) {
-        Ccur[0] = N - N / 2;
-        Cnxt[0] = N / 2;
-    }
-    __syncwarp();
-    const bool own_c0 = lane == 0;  // the lane whose k = lane + 32q is 0 at q = 0
-    // correlation masks of the recomputation: i < N - k for k = lane + 32q
-    uint32_t cmask[kRecompute ? NW : 1][kRecompute ? NW : 1];
-    int32_t nk[NW];
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-        const int k = lane + 32 * q;
-        nk[q] = (k >= 1 && k <= N - 1) ? N - k : 0;
-        if constexpr (kRecompute) {
-#pragma unroll
-            for (int w = 0; w + q < NW; ++w) cmask[q][w] = word_lowmask(w, nk[q]);
+        for (int q = 0; q < NW; ++q) {
+            const int j = lane + 32 * q;
+            s[q] = j < N ? ((XB[q] & 1u) ? 1 : -1) : 0;
+            C0[j] = c[q];
+            C0[-j] = c[q];
+            S0[j] = static_cast<int8_t>(-2 * s[q]);
+            S0[j - NB] = 0;
+            S0[j + NB] = 0;
         }
-    }
-    // all-ones masks: bits 0 .. N-1, and every bit (the move's ranges below)
-    uint32_t allN[NW], allB[NW];
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        allN[w] = word_lowmask(w, N);
-        allB[w] = kFull;
-    }
-    const int min_t = max_iter / 10;
-    const int max_t = (12 * max_iter) / 100;
-    const int64_t nsteps = budget < 0 ? max_iter : (budget < max_iter ? budget : max_iter);
-    uint32_t rx = 0, ry = 0;
-    int64_t steps = 0;
-    bool fault = false;
-
-    for (int t = 1; t <= nsteps; ++t) {
-        if (((t - 1) & 31) == 0) {  // draws of steps t .. t+31, one per lane
-            const uint4 r = draw4(key, inst, g, static_cast<uint32_t>(t + lane), kPurposeStep);
-            rx = r.x;
-            ry = r.y;
-        }
-        const int src = (t - 1) & 31;
-        const uint32_t u_tie = __shfl_sync(kFull, rx, src);
-        const uint32_t u_ten = __shfl_sync(kFull, ry, src);
-        // ---- E_j for j = lane + 32q, admissibility, packed (E_j, j) keys
-        const int32_t E0 = E + 4 * (N - 1);
-        int32_t cand[NW], Mq[NW];
-        int32_t kmin_l = INT_MAX;
-#pragma unroll
-        for (int q = QB; q < QE; ++q) {
-            int dm = 0;
-#pragma unroll
-            for (int w = 0; w <= q && w + q < NW; ++w)
-                dm += __popc((XB[q + w] ^ YB[w + NW - 1 - q]) & mmask[q][w]);
-            Mq[q] = Lq[q] - 2 * dm;
-            // s_j R_j (bit 0 of X_j is b_j): a select for two-word sequences,
-            // a multiply by 2 b_j - 1 above (off the busy ALU pipe; 3-6 % less
-            // time per launch for N = 92 .. 200 on GB300, 1 % more at N = 64)
-            int32_t sR;
-            if constexpr (NW >= 3)
-                sR = (2 * static_cast<int32_t>(XB[q] & 1u) - 1) * R[q];
-            else
-                sR = (XB[q] & 1u) ? R[q] : -R[q];
-            const int32_t Ej = E0 + 8 * Mq[q] - 4 * sR;
-            const bool adm = ((jvalid >> q) & 1u) && (tabu[q] < t || Ej < E_best);
-            cand[q] = adm ? Ej : INT_MAX;
-            // E_j < 2^23 for N <= 256 and j < 256: (E_j, j) packs into 31 bits
-            kmin_l = min(kmin_l, adm ? (Ej << 8) | (lane + 32 * q) : INT_MAX);
-        }
-        const int32_t kmin_w = __reduce_min_sync(kFull, kmin_l);
-        int eq = 0;  // this warp's admissible minimisers
-#pragma unroll
-        for (int q = QB; q < QE; ++q) eq += (cand[q] == (kmin_w >> 8)) ? 1 : 0;
-        const int count_w = __reduce_add_sync(kFull, eq);  // 0 when nothing is admissible
-        int32_t kmin = kmin_w;
-        int count = count_w, count_lo = 0;  // count_lo: minimisers of the lower half (WPS = 2)
-        if constexpr (WPS == 2) {
-            uint64_t o = 0;
-            if (!pair_exchange(link, HALF, (*xseq)++,
-                               (static_cast<uint64_t>(count_w) << 31) | static_cast<uint32_t>(kmin_w), o, lane)) {
-                fault = true;
-                break;
-            }
-            const int32_t kmin_o = static_cast<int32_t>(o & 0x7FFFFFFFu);
-            const int count_o = static_cast<int>(o >> 31);
-            kmin = min(kmin_w, kmin_o);
-            // minimisers of either half: the same energy, whatever their index
-            const int cw = (kmin_w >> 8) == (kmin >> 8) ? count_w : 0;
-            const int co = (kmin_o >> 8) == (kmin >> 8) ? count_o : 0;
-            count = cw + co;
-            count_lo = HALF == 0 ? cw : co;
-        }
-        // Every move tabu and none aspirating: the search has no admissible
-        // move and stops.  The default maxIter keeps maxTabu below N, so only a
-        // user maxIter of about 8N or more (maxTabu >= N) gets here.
-        if (kmin == INT_MAX) break;
-        const int32_t m = kmin >> 8;
-        int p = kmin & 255;  // lowest admissible minimiser
-        {
-            int idx = count > 1 ? static_cast<int>((static_cast<uint64_t>(u_tie) * count) >> 32) : 0;
-            if (idx > 0) {  // the idx-th minimiser in ascending j
-                bool mine = true;  // WPS = 2: the warp holding it finds it, then tells the other
-                if constexpr (WPS == 2) {
-                    mine = HALF == 0 ? idx < count_lo : idx >= count_lo;
-                    if (HALF == 1) idx -= count_lo;
-                }
-                if (mine) {
-                    bool found = false;
-#pragma unroll
-                    for (int q = QB; q < QE; ++q) {
-                        const uint32_t tb = __ballot_sync(kFull, cand[q] == m);
-                        const int pc_q = __popc(tb);
-                        if (!found) {
-                            if (idx < pc_q) {
-                                p = 32 * q + nth_set_bit(tb, idx);
-                                found = true;
-                            } else {
-                                idx -= pc_q;
-                            }
-                        }
-                    }
-                }
-                if constexpr (WPS == 2) {
-                    uint64_t o = 0;
-                    if (!pair_exchange(link, HALF, (*xseq)++, mine ? static_cast<uint64_t>(p) : 0u, o, lane)) {
-                        fault = true;
-                        break;
-                    }
-                    if (!mine) p = static_cast<int>(o);
-                }
-            }
-        }
-        // ---- the move p: its windows (before the flip; bits k >= 1 are the
-        // same after it), s_p, and the ranges k in [1, N-1-p] and [1, p]
-        uint32_t Xp[NW], Yp[NW], mu[NW], mv[NW];
-        shr_uniform2<NW>(B, allN, p, Xp, mu);            // mu: bits 0 .. N-1-p
-        shr_uniform2<NW>(RL, allB, NB - 1 - p, Yp, mv);  // mv: bits 0 .. p
-        mu[0] &= ~1u;
-        mv[0] &= ~1u;
-        const int32_t sp2 = (Xp[0] & 1u) ? 2 : -2;  // 2 s_p
-        int32_t dq[NW], c0[NW];
-#pragma unroll
-        for (int q = QB; q < QE; ++q) {
-            dq[q] = abs(p - (lane + 32 * q));
-            c0[q] = Ccur[dq[q]];  // C_d before the move
-        }
-        flip_bit<NW>(B, p);
-        // the mirror image: one bit flip for two words (a 64-bit one-hot), a
-        // full reversal (one brev per word, no per-word select) above
-        if constexpr (NW >= 3)
-            reverse_bits<NW>(B, RL);
-        else
-            flip_bit<NW>(RL, NB - 1 - p);
-        pivot_windows<NW>(B, RL, lane, XB, YB);
-        if constexpr (kRecompute) {
-#pragma unroll
-            for (int q = 0; q < NW; ++q) {
-                int cnt = 0;
-#pragma unroll
-                for (int w = 0; w + q < NW; ++w) cnt += __popc((B[w] ^ XB[w + q]) & cmask[q][w]);
-                c[q] = nk[q] - 2 * cnt;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < NW; ++q) {
-                const int32_t bx = (Xp[q] >> lane) & 1u, by = (Yp[q] >> lane) & 1u;
-                const int32_t sx = ((mu[q] >> lane) & 1u) ? 2 * bx - 1 : 0;
-                const int32_t sy = ((mv[q] >> lane) & 1u) ? 2 * by - 1 : 0;
-                c[q] -= sp2 * (sx + sy);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < NW; ++q)
-            if (q > 0 || !own_c0) Cnxt[lane + 32 * q] = c[q];
         __syncwarp();
 #pragma unroll
         for (int q = QB; q < QE; ++q) {
             const int j = lane + 32 * q;
-            const int32_t c1 = Cnxt[dq[q]];  // C'_d
-            // crossed pairs: (p+k, j-k) for k <= min(N-1-p, j) and
-            // (p-k, j+k) for k <= min(p, N-1-j); each disagreement is -1
-            uint32_t words[NW + 1];
-#pragma unroll
-            for (int w = 0; w <= q; ++w)
-                words[w] = (Xp[w] ^ YB[w + NW - 1 - q]) & mu[w] & (w == q ? low_l : kFull);
-#pragma unroll
-            for (int w = 0; w + q < NW; ++w) words[q + 1 + w] = (Yp[w] ^ XB[q + w]) & mv[w] & mX[q + w];
-            const int32_t F = min(N - 1 - p, j) + min(p, N - 1 - j) - 2 * csa_popc<NW + 1, 1>(words);
-            const int32_t sj2 = (XB[q] & 1u) ? 2 : -2;  // 2 s'_j
-            R[q] -= sp2 * (c0[q] + c1 + F) + sj2;
+            // D_j / 4 = N - 1 + 2 M_j - s_j R_j, 2 M_j = V_{2j} - 1
+            const int32_t d4 = N - 2 + Vs[2 * j] - s[q] * (2 * S[q] - T[q]);
+            K[q] = j < N ? d4 * (kLow + 1) + 2 * j + (s[q] > 0 ? 1 : 0) : kNone;
+            tabu[q] = 0;
         }
-        {
-            int32_t* tmp = Ccur;
-            Ccur = Cnxt;
-            Cnxt = tmp;
-        }
-        const int32_t expiry = t + rand_int(min_t, max_t, u_ten);
+        __syncwarp();
+    }
+    uint32_t Bb[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) Bb[w] = seq[w];
+    const int min_t = max_iter / 10;
+    const int max_t = (12 * max_iter) / 100;
+    const int nsteps = static_cast<int>(budget < 0 ? max_iter : (budget < max_iter ? budget : max_iter));
+    // Every D_j / 4 loses 4 per move besides the terms below; the keys leave
+    // that out, so a stored key is the true one + off, off = 4 << 9 per move
+    // since the last multiple of 32.  thr (stored likewise): a key below it is
+    // a move to below E_best, (E_best - E) / 4 << 9.
+    constexpr int32_t kDrift = 4 * (kLow + 1);
+    int32_t off = 0, thr = 0;
+    int t = 0;  // moves made; this step is t + 1
+    bool fault = false, stuck = false;
+    const int32_t* const Vl = Vs + lane;
+    const int32_t* const Cl = C0 + lane;
+    const int8_t* const Al = S0 + 2 * lane;
+    const int8_t* const Bl = S0 - lane;
+
+    while (t < nsteps && !fault && !stuck) {
+        // draws of steps t+1 .. t+32, one per lane: tie pick, and expiry of the move's tabu
+        const uint4 r = draw4(key, inst, g, static_cast<uint32_t>(t + 1 + lane), kPurposeStep);
+        const uint32_t u_tie_l = r.x;
+        const int32_t expiry_l = t + 1 + lane + rand_int(min_t, max_t, r.y);
 #pragma unroll
         for (int q = QB; q < QE; ++q)
-            if (lane + 32 * q == p) tabu[q] = expiry;
-        E = m;
-        if (m < E_best) {
-            E_best = m;
+            if (K[q] != kNone) K[q] -= off;
+        thr -= off;
+        off = 0;
+        const int tend = min(t + 32, nsteps);
+#pragma unroll 1
+        for (; t < tend; ++t) {
+            // ---- admissible minimum
+            int32_t cand[NW];
+            int32_t kmin_l = kNone;
 #pragma unroll
-            for (int w = 0; w < NW; ++w) Bb[w] = B[w];
-        }
-        ++steps;
-        if constexpr (TRACE) {
-            if (trace_len < trace_cap) {
-                if (lane == 0 && HALF == 0) trace[trace_len] = make_int4(static_cast<int>(g), t, p, m);
-                ++trace_len;
+            for (int q = QB; q < QE; ++q) {
+                bool adm = tabu[q] <= t || K[q] < thr;
+                if (FIX_FIRST && q == 0) adm = adm && lane != 0;
+                cand[q] = adm ? K[q] : kNone;
+                kmin_l = min(kmin_l, cand[q]);
+            }
+            const int32_t kmin_w = __reduce_min_sync(kFull, kmin_l);
+            int32_t kmin = kmin_w;
+            bool tie = false;  // another admissible move is as good
+            int count_w = 0, count = 0, count_lo = 0;  // count_lo: minimisers of the lower half (WPS = 2)
+            if constexpr (WPS == 1) {
+                // least distance above the minimum itself; the same energy within kLow
+                uint32_t above = 0xFFFFFFFFu;
+#pragma unroll
+                for (int q = 0; q < NW; ++q)
+                    above = min(above, static_cast<uint32_t>(cand[q]) - static_cast<uint32_t>(kmin_w) - 1u);
+                tie = __any_sync(kFull, above < static_cast<uint32_t>(kLow - (kmin_w & kLow))) || kmin_w == kNone;
+            } else {
+#pragma unroll
+                for (int q = QB; q < QE; ++q) count_w += __popc(__ballot_sync(kFull, cand[q] <= (kmin_w | kLow)));
+                // a key is above -2^30: shifted, it fits 31 bits beside the count
+                const uint32_t kx = kmin_w == kNone ? 0x7FFFFFFFu : static_cast<uint32_t>(kmin_w + (1 << 30));
+                uint64_t o = 0;
+                if (!pair_exchange(link, HALF, (*xseq)++, (static_cast<uint64_t>(count_w) << 31) | kx, o, lane)) {
+                    fault = true;
+                    break;
+                }
+                const uint32_t ko = static_cast<uint32_t>(o & 0x7FFFFFFFu);
+                const int32_t kmin_o = ko == 0x7FFFFFFFu ? kNone : static_cast<int32_t>(ko) - (1 << 30);
+                const int count_o = static_cast<int>(o >> 31);
+                kmin = min(kmin_w, kmin_o);
+                // minimisers of either half: the same energy, whatever their index
+                const int cw = kmin_w <= (kmin | kLow) ? count_w : 0;
+                const int co = kmin_o <= (kmin | kLow) ? count_o : 0;
+                count = cw + co;
+                count_lo = HALF == 0 ? cw : co;
+                tie = count > 1;
+            }
+            int klow = kmin & kLow;  // 2p + (s_p == +1), p the lowest admissible minimiser
+            // ---- the move's V, C and mirror spins (times -2), and what they
+            // make of the keys, V and C, for the lowest minimiser: done before
+            // the ties are looked at, and again if one of the others is taken
+            int32_t kn[NW], vn[NW], cn[NW];
+            auto score_move = [&](const int klow) {
+                const int p = klow >> 1;
+                const int32_t sp = 2 * (klow & 1) - 1;
+#pragma unroll
+                for (int q = 0; q < NW; ++q) {
+                    const int32_t v = Vl[p + 32 * q];
+                    const int32_t cd = Cl[32 * q - p];
+                    const int32_t sb = Bl[2 * p - 32 * q];
+                    cn[q] = cd + sp * (sb - 2 * s[q]);
+                    vn[q] = v - 4 * sp * s[q];
+                    if (q >= QB && q < QE)
+                        kn[q] = K[q] + (2 * (kLow + 1) * sp) * (s[q] * (cd + cn[q] + v) + Al[64 * q - p]);
+                }
+            };
+            const int32_t expiry = __shfl_sync(kFull, expiry_l, t);
+            bool again;
+            do {
+                again = false;
+                score_move(klow);
+                if (tie) {
+                    tie = false;
+                    // Every move tabu and none aspirating: the search has no admissible
+                    // move and stops.  The default maxIter keeps maxTabu below N, so only a
+                    // user maxIter of about 8N or more (maxTabu >= N) gets here.
+                    if (kmin == kNone) {
+                        stuck = true;
+                        break;
+                    }
+                    uint32_t tb[NW];
+    #pragma unroll
+                    for (int q = QB; q < QE; ++q) {
+                        tb[q] = __ballot_sync(kFull, cand[q] <= (kmin | kLow));
+                        if constexpr (WPS == 1) count += __popc(tb[q]);
+                    }
+                    const uint32_t u_tie = __shfl_sync(kFull, u_tie_l, t);
+                    int idx = static_cast<int>((static_cast<uint64_t>(u_tie) * count) >> 32);
+                    if (idx > 0) {  // the idx-th minimiser in ascending j
+                        int p = 0;
+                        bool mine = true;  // WPS = 2: the warp holding it finds it, then tells the other
+                        if constexpr (WPS == 2) {
+                            mine = HALF == 0 ? idx < count_lo : idx >= count_lo;
+                            if (HALF == 1) idx -= count_lo;
+                        }
+                        if (mine) {
+                            bool found = false;
+    #pragma unroll
+                            for (int q = QB; q < QE; ++q) {
+                                const int pc_q = __popc(tb[q]);
+                                if (!found) {
+                                    if (idx < pc_q) {
+                                        p = 32 * q + nth_set_bit(tb[q], idx);
+                                        found = true;
+                                    } else {
+                                        idx -= pc_q;
+                                    }
+                                }
+                            }
+                        }
+                        if constexpr (WPS == 2) {
+                            uint64_t o = 0;
+                            if (!pair_exchange(link, HALF, (*xseq)++, mine ? static_cast<uint64_t>(p) : 0u, o, lane)) {
+                                fault = true;
+                                break;
+                            }
+                            if (!mine) p = static_cast<int>(o);
+                        }
+                        klow = 2 * p + (S0[p] < 0 ? 1 : 0);
+                        if constexpr (kRecompute)
+                            score_move(klow);
+                        else
+                            again = true;
+                    }
+                }
+            } while (again);
+            if (stuck || fault) break;
+            __syncwarp();  // every lane has read what the stores below change
+            // ---- apply the move
+            const int p = klow >> 1;
+            const int32_t sp = 2 * (klow & 1) - 1;
+            const int32_t dk = kmin & ~kLow;
+            off += kDrift;
+            {
+                int32_t* const vp = Vs + lane + p;
+                int32_t* const cp = C0 + lane - p;
+                int32_t* const cm = C0 - lane + p;
+                // D'_p = -D_p and s'_p = -s_p: (off - kDrift - dk) + off, the spin bit flipped
+                const int32_t kp = 2 * off - kDrift - dk + (klow ^ 1);
+#pragma unroll
+                for (int q = 0; q < NW; ++q) {
+                    const bool own = p - lane == 32 * q;
+                    if (q >= QB && q < QE) {
+                        K[q] = own ? kp : kn[q];
+                        tabu[q] = own ? expiry : tabu[q];
+                    }
+                    if (!own) vp[32 * q] = vn[q];
+                    cp[32 * q] = cn[q];
+                    cm[-32 * q] = cn[q];
+                    if (own) s[q] = -s[q];
+                }
+                S0[p] = static_cast<int8_t>(2 * sp);  // every lane the same byte
+            }
+            __syncwarp();
+            const int32_t gain = thr - dk;  // (E_best - E') / 4 << 9
+            thr = min(gain, 0) + off;
+            if (gain > 0) {
+                E_best -= gain >> 7;  // 4 (E_best - E') / 4
+#pragma unroll
+                for (int w = 0; w < NW; ++w) Bb[w] = __ballot_sync(kFull, s[w] > 0);
+            }
+            if constexpr (TRACE) {
+                if (trace_len < trace_cap) {
+                    // E' = E_best - (E_best - E')
+                    if (lane == 0 && HALF == 0)
+                        trace[trace_len] = make_int4(static_cast<int>(g), t + 1, p, E_best - (min(gain, 0) >> 7));
+                    ++trace_len;
+                }
             }
         }
     }
-    __syncwarp();  // the buffers are reused by the caller
+    __syncwarp();  // the scratch is reused by the caller
 #pragma unroll
     for (int w = 0; w < NW; ++w) seq[w] = Bb[w];
     TabuOut out;
-    out.steps = steps;
+    out.steps = t;
     out.E_best = E_best;
     out.fault = fault;
     return out;
