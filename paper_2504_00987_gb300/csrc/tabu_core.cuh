@@ -324,6 +324,72 @@ __device__ __forceinline__ void store_self_convolution(const uint32_t (&B)[NW], 
     }
 }
 
+// The scratch's parts: V_m, m = 0 .. 2 NB - 1; C_d at C[d] and C[-d]; -2 s~_i
+// at S[i], i = -NB .. 2 NB - 1.
+template <int NW>
+struct TabuScratch {
+    int32_t* V;
+    int32_t* C;
+    int8_t* S;
+    __device__ __forceinline__ explicit TabuScratch(int32_t* base)
+        : V(base), C(base + 3 * 32 * NW), S(reinterpret_cast<int8_t*>(base + 4 * 32 * NW) + 32 * NW) {}
+};
+
+// Fills the scratch for a search from `seq` and returns its energy; s[q] is
+// the spin (0 for j >= N) and d4[q] the energy change D_j / 4 of the lane's
+// j = lane + 32q (unset for j >= N).
+template <int NW>
+__device__ __forceinline__ int32_t search_setup(const uint32_t (&seq)[NW], int N, int lane,
+                                                int32_t* __restrict__ Cs, int32_t (&s)[NW], int32_t (&d4)[NW]) {
+    constexpr int NB = 32 * NW;
+    const TabuScratch<NW> sh(Cs);
+    int32_t c[NW];
+    correlations<NW>(seq, N, lane, c);
+    int32_t sq = 0;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) sq += c[q] * c[q];
+    const int32_t E = __reduce_add_sync(kFull, sq);
+    // R_j = 2 S_j - T_j from the bit planes of C_k (S_j) and the prefix sums
+    // of C_k (T_j = PC(j) + PC(N-1-j))
+    uint32_t RL[NW], XB[NW], YB[NW], par[NW];
+    reverse_bits<NW>(seq, RL);
+    pivot_windows<NW>(seq, RL, lane, XB, YB);
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const uint32_t alt = ((N - 32 * w) & 1) ? 0x55555555u : 0xAAAAAAAAu;  // (N - k) odd
+        par[w] = alt & word_lowmask(w, N) & (w == 0 ? ~1u : kFull);
+    }
+    uint32_t X[NW][NW], Y[NW][NW];
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+#pragma unroll
+        for (int w = 0; w + q < NW; ++w) X[q][w] = XB[q + w];
+#pragma unroll
+        for (int w = 0; w <= q; ++w) Y[q][w] = YB[w + NW - 1 - q];
+    }
+    int32_t S[NW], pc[NW], T[NW];
+    score_dispatch<NW>(plane_count<NW>(c), c, par, X, Y, S);
+    prefix_own<NW>(c, lane, pc);
+    mirror_terms<NW>(pc, N, lane, Cs, T);
+    store_self_convolution<NW>(seq, RL, N, lane, sh.V);
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+        const int j = lane + 32 * q;
+        s[q] = j < N ? ((XB[q] & 1u) ? 1 : -1) : 0;
+        sh.C[j] = c[q];
+        sh.C[-j] = c[q];
+        sh.S[j] = static_cast<int8_t>(-2 * s[q]);
+        sh.S[j - NB] = 0;
+        sh.S[j + NB] = 0;
+    }
+    __syncwarp();
+    // D_j / 4 = N - 1 + 2 M_j - s_j R_j, 2 M_j = V_{2j} - 1
+#pragma unroll
+    for (int q = 0; q < NW; ++q) d4[q] = N - 2 + sh.V[2 * (lane + 32 * q)] - s[q] * (2 * S[q] - T[q]);
+    __syncwarp();
+    return E;
+}
+
 // One tabu search from `seq` (warp-uniform).  On return `seq` holds
 // bestSeqTS.  Draws: step t uses Philox(instance, g, t, 4): x tie, y tenure.
 // FIX_FIRST: bit 0 (s_1) is never a candidate move.
@@ -399,63 +465,17 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     constexpr bool kRecompute = NW <= 4 ? NW > 2 : true;
     constexpr int32_t kLow = 511;  // key bits below the energy change
     constexpr int32_t kNone = INT_MAX & ~kLow;  // no candidate: above every key, low bits those of j = 0
-    int32_t* const Vs = Cs;                                     // V_m, m = 0 .. 2 NB - 1
-    int32_t* const C0 = Cs + 3 * NB;                            // C_d at C0[d] and C0[-d]
-    int8_t* const S0 = reinterpret_cast<int8_t*>(Cs + 4 * NB) + NB;  // -2 s~_i, i = -NB .. 2 NB - 1
-    int32_t s[NW], c[NW];
-    correlations<NW>(seq, N, lane, c);
-    int32_t E_best;
-    {
-        int32_t sq = 0;
+    const TabuScratch<NW> sh(Cs);
+    int32_t* const Vs = sh.V;
+    int32_t* const C0 = sh.C;
+    int8_t* const S0 = sh.S;
+    int32_t s[NW], K[NW], tabu[NW];
+    int32_t E_best = search_setup<NW>(seq, N, lane, Cs, s, K);
 #pragma unroll
-        for (int q = 0; q < NW; ++q) sq += c[q] * c[q];
-        E_best = __reduce_add_sync(kFull, sq);
-    }
-    // R_j = 2 S_j - T_j from the bit planes of C_k (S_j) and the prefix sums
-    // of C_k (T_j = PC(j) + PC(N-1-j)), once per search.
-    int32_t K[NW], tabu[NW];
-    {
-        uint32_t RL[NW], XB[NW], YB[NW], par[NW];
-        reverse_bits<NW>(seq, RL);
-        pivot_windows<NW>(seq, RL, lane, XB, YB);
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const uint32_t alt = ((N - 32 * w) & 1) ? 0x55555555u : 0xAAAAAAAAu;  // (N - k) odd
-            par[w] = alt & word_lowmask(w, N) & (w == 0 ? ~1u : kFull);
-        }
-        uint32_t X[NW][NW], Y[NW][NW];
-#pragma unroll
-        for (int q = 0; q < NW; ++q) {
-#pragma unroll
-            for (int w = 0; w + q < NW; ++w) X[q][w] = XB[q + w];
-#pragma unroll
-            for (int w = 0; w <= q; ++w) Y[q][w] = YB[w + NW - 1 - q];
-        }
-        int32_t S[NW], pc[NW], T[NW];
-        score_dispatch<NW>(plane_count<NW>(c), c, par, X, Y, S);
-        prefix_own<NW>(c, lane, pc);
-        mirror_terms<NW>(pc, N, lane, Cs, T);
-        store_self_convolution<NW>(seq, RL, N, lane, Vs);
-#pragma unroll
-        for (int q = 0; q < NW; ++q) {
-            const int j = lane + 32 * q;
-            s[q] = j < N ? ((XB[q] & 1u) ? 1 : -1) : 0;
-            C0[j] = c[q];
-            C0[-j] = c[q];
-            S0[j] = static_cast<int8_t>(-2 * s[q]);
-            S0[j - NB] = 0;
-            S0[j + NB] = 0;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int q = QB; q < QE; ++q) {
-            const int j = lane + 32 * q;
-            // D_j / 4 = N - 1 + 2 M_j - s_j R_j, 2 M_j = V_{2j} - 1
-            const int32_t d4 = N - 2 + Vs[2 * j] - s[q] * (2 * S[q] - T[q]);
-            K[q] = j < N ? d4 * (kLow + 1) + 2 * j + (s[q] > 0 ? 1 : 0) : kNone;
-            tabu[q] = 0;
-        }
-        __syncwarp();
+    for (int q = QB; q < QE; ++q) {
+        const int j = lane + 32 * q;
+        K[q] = j < N ? K[q] * (kLow + 1) + 2 * j + (s[q] > 0 ? 1 : 0) : kNone;
+        tabu[q] = 0;
     }
     uint32_t Bb[NW];
 #pragma unroll
