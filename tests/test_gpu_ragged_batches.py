@@ -1,0 +1,47 @@
+"""Batches whose size is ragged against what a warp or a CTA takes at once, at
+lengths on either side of each word count, against the oracle (exact)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+NS = [3, 4, 16, 31, 32, 33, 47, 64, 65, 80, 96, 97, 128, 130, 161, 192, 224, 225, 256]
+
+
+@pytest.fixture(scope="module")
+def labs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_2504_00987_gb300 as labs
+
+    return labs
+
+
+def sequences(N, B, dirty):
+    """Random rows and the extreme ones; `dirty` sets the bits beyond N, which every call ignores."""
+    from paper_2504_00987_gb300 import workloads
+
+    a = np.concatenate([workloads.sequence_edge_cases(N), workloads.random_sequences(N, B, seed=B + N)])[:B]
+    if dirty and N % 64:
+        a = a.copy()
+        a[:, -1] |= np.uint64((1 << 64) - (1 << (N % 64)))
+    return a
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a).view(np.int64)).cuda()
+
+
+@pytest.mark.parametrize("B", [1, 7, 33, 130])
+@pytest.mark.parametrize("N", NS)
+def test_skew_deviation(labs, orc, N, B):
+    a = sequences(N, B, dirty=True)
+    got = labs.skew_deviation_batch(dev(a), N).cpu().numpy()
+    clean = sequences(N, B, dirty=False)
+    for b in range(B):
+        assert got[b] == orc.skew_deviation(clean[b], N)
