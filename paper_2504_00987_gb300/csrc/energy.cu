@@ -1,78 +1,148 @@
 // energy.cu -- labs_energy_batch: C_k (Eq. 1) and E (Eq. 2) of B packed
 // sequences.  C_k = (N - k) - 2 popc(b_i xor b_{i+k}, i < N - k): one
 // funnel-shifted window, an xor and a popcount per 32 products.
-//  - E only: one thread per sequence (W words in registers), reads W*8 B
-//    and writes 4 B per sequence.
-//  - E and C: one warp per sequence, lane l computes C_k for k = l + 32q,
-//    so each row of C is written by consecutive lanes (coalesced).
+//  - E only, many sequences: one thread per sequence (NW words in registers).
+//  - E and C, or few sequences: one warp per sequence, lane l computes C_k for
+//    k = l + 32q, so each row of C is written by consecutive lanes
+//    (coalesced); the masks of a lane are those of every sequence, so a warp
+//    keeps them and takes one sequence after the other.
+// What bounds them: popcounts, 8 cycles of the XU pipe a warp and 8 of them per
+// 32 values of k at N = 120 after the full adders (10 words), 51 us for 10^6
+// sequences; with C, the stores of its rows (16-byte stores through shared
+// memory took 35 us where these take 33).  On GB300, N = 120: 10^6 energies
+// 56 us (masks rebuilt for every word and round, no adders: 151), 300,000 with
+// C 33 us, 4.3 TB/s (57); 100 energies 2.0 us on the device (8.8).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
+#include "capi_util.h"
 #include "kernels.h"
 #include "tabu_core.cuh"
 
 namespace lgpu {
 
+constexpr int kEnergyThreads = 256;
+
+// Words per row in memory: whole 64-bit words.
 template <int NW>
-__global__ void __launch_bounds__(256) energy_thread_kernel(const uint32_t* __restrict__ seqs, int N,
-                                                            int64_t B, int32_t* __restrict__ E) {
+constexpr int kRowWords = (NW + 1) & ~1;
+
+template <int NW>
+__device__ __forceinline__ void load_row(const uint32_t* __restrict__ seqs, int64_t b, int N, uint32_t (&s)[NW]) {
+    const uint2* src = reinterpret_cast<const uint2*>(seqs + b * kRowWords<NW>);  // 8-byte aligned rows
+#pragma unroll
+    for (int v = 0; v < kRowWords<NW> / 2; ++v) {
+        const uint2 x = __ldg(src + v);
+        s[2 * v] = x.x;
+        if (2 * v + 1 < NW) s[2 * v + 1] = x.y;
+    }
+    s[NW - 1] &= word_lowmask(NW - 1, N);  // bits >= N are ignored
+}
+
+template <int NW>
+__global__ void __launch_bounds__(kEnergyThreads) energy_thread_kernel(const uint32_t* __restrict__ seqs, int N,
+                                                                       int64_t B, int32_t* __restrict__ E) {
     const int64_t b = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (b >= B) return;
     uint32_t s[NW];
-    const uint2* src = reinterpret_cast<const uint2*>(seqs + b * NW);  // 8-byte aligned rows
-#pragma unroll
-    for (int v = 0; v < NW / 2; ++v) {
-        const uint2 x = __ldg(src + v);
-        s[2 * v] = x.x;
-        s[2 * v + 1] = x.y;
-    }
-#pragma unroll
-    for (int w = 0; w < NW; ++w) s[w] &= word_lowmask(w, N);
-    E[b] = thread_energy<NW>(s, N);
+    load_row<NW>(seqs, b, N, s);
+    E[b] = thread_energy<NW, true>(s, N);
 }
 
-template <int NW>
-__global__ void __launch_bounds__(256) energy_warp_kernel(const uint32_t* __restrict__ seqs, int N,
-                                                          int64_t B, int32_t* __restrict__ E,
-                                                          int32_t* __restrict__ C) {
+// C_k of the lane's k = lane + 32q.
+template <int NW, int q = 0>
+__device__ __forceinline__ void lane_correlations(const uint32_t (&s)[NW], const uint32_t (&mask)[NW], int N, int lane,
+                                                  int32_t (&c)[NW]) {
+    if constexpr (q < NW) {
+        c[q] = max(N - lane - 32 * q, 0) - 2 * unequal_pairs<NW, q>(s, mask, lane);
+        lane_correlations<NW, q + 1>(s, mask, N, lane, c);
+    }
+}
+
+// A warp takes ROWS consecutive sequences at a time, so that one's loads and
+// reduction overlap the others' work.
+template <int NW, int ROWS>
+__global__ void __launch_bounds__(kEnergyThreads) energy_warp_kernel(const uint32_t* __restrict__ seqs, int N,
+                                                                     int64_t B, int32_t* __restrict__ E,
+                                                                     int32_t* __restrict__ C) {
     const int lane = threadIdx.x & 31;
-    const int64_t b = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    if (b >= B) return;
-    uint32_t s[NW];
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (kEnergyThreads / 32);
+    const int64_t warp = (static_cast<int64_t>(blockIdx.x) * kEnergyThreads + threadIdx.x) >> 5;
+    uint32_t mask[NW];
+    pair_masks<NW, false>(N, lane, mask);
+    for (int64_t b0 = warp * ROWS; b0 < B; b0 += warps * ROWS) {
+        const int rows = static_cast<int>(min(static_cast<int64_t>(ROWS), B - b0));
+        int32_t sq[ROWS];
 #pragma unroll
-    for (int w = 0; w < NW; ++w) s[w] = __ldg(seqs + b * NW + w) & word_lowmask(w, N);
-    int32_t c[NW];
-    correlations<NW>(s, N, lane, c);
-    int32_t sq = 0;
+        for (int r = 0; r < ROWS; ++r) {
+            uint32_t s[NW];
+            load_row<NW>(seqs, min(b0 + r, B - 1), N, s);
+            int32_t c[NW];
+            lane_correlations<NW>(s, mask, N, lane, c);
+            sq[r] = lane >= 1 ? c[0] * c[0] : 0;  // C_0 does not count
 #pragma unroll
-    for (int q = 0; q < NW; ++q) {
-        sq += c[q] * c[q];
-        const int k = lane + 32 * q;
-        if (k >= 1 && k <= N - 1) C[b * (N - 1) + (k - 1)] = c[q];
+            for (int q = 1; q < NW; ++q) sq[r] += c[q] * c[q];
+            if (C != nullptr && r < rows) {
+#pragma unroll
+                for (int q = 0; q < NW; ++q) {
+                    const int k = lane + 32 * q;
+                    if (k >= 1 && k <= N - 1) C[(b0 + r) * (N - 1) + k - 1] = c[q];
+                }
+            }
+        }
+        int32_t e = 0;
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int32_t t = __reduce_add_sync(kFull, sq[r]);
+            e = lane == r ? t : e;
+        }
+        if (lane < rows) E[b0 + lane] = e;
     }
-    sq = __reduce_add_sync(kFull, sq);
-    if (lane == 0) E[b] = sq;
 }
 
+template <int NW, int ROWS>
+static void launch_energy_warps(const uint32_t* seqs, int N, int64_t B, int32_t* d_E, int32_t* d_C,
+                                cudaStream_t stream) {
+    constexpr int per_block = kEnergyThreads / 32 * ROWS;
+    const int64_t wave = static_cast<int64_t>(lcapi::sm_count()) * 8;  // 64 warps on every SM
+    const int64_t blocks = std::min((B + per_block - 1) / per_block, wave);
+    energy_warp_kernel<NW, ROWS><<<static_cast<unsigned>(blocks), kEnergyThreads, 0, stream>>>(seqs, N, B, d_E, d_C);
+}
+
+// E alone takes a thread per sequence from 8 NW^2 sequences per SM on: a
+// thread's chain grows with NW^2, and below that it outlasts the warps'
+// (us, warps / threads: N = 64 1.8 / 2.4 at B = 4,000, 3.0 / 2.5 at 20,000;
+// N = 120 2.9 / 3.8 at 10,000, 5.5 / 5.9 at 40,000, 24 / 18 at 300,000;
+// N = 256 12 / 17 at 40,000, 25 / 24 at 100,000).  A warp
+// takes one sequence at a time up to 32 per SM, four from there (E and C at
+// N = 120: 2.0 / 2.5 at 1,000, 5.5 / 4.4 at 20,000).
 template <int NW>
 static cudaError_t launch_energy_w(const uint64_t* d_seqs, int N, int64_t B, int32_t* d_E,
                                    int32_t* d_C, cudaStream_t stream) {
     const uint32_t* seqs = reinterpret_cast<const uint32_t*>(d_seqs);
-    if (d_C == nullptr) {
-        const int64_t blocks = (B + 255) / 256;
-        energy_thread_kernel<NW><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(seqs, N, B, d_E);
+    const int64_t sms = lcapi::sm_count();
+    if (d_C == nullptr && B > sms * 8 * NW * NW) {
+        const int64_t blocks = (B + kEnergyThreads - 1) / kEnergyThreads;
+        energy_thread_kernel<NW><<<static_cast<unsigned>(blocks), kEnergyThreads, 0, stream>>>(seqs, N, B, d_E);
+    } else if (B <= sms * 32) {
+        launch_energy_warps<NW, 1>(seqs, N, B, d_E, d_C, stream);
     } else {
-        const int64_t blocks = (B + 7) / 8;
-        energy_warp_kernel<NW><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(seqs, N, B, d_E, d_C);
+        launch_energy_warps<NW, 4>(seqs, N, B, d_E, d_C, stream);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_energy(const uint64_t* d_seqs, int N, int64_t B, int32_t* d_E, int32_t* d_C,
                           cudaStream_t stream) {
-    switch ((N + 63) / 64) {
-        case 1: return launch_energy_w<2>(d_seqs, N, B, d_E, d_C, stream);
-        case 2: return launch_energy_w<4>(d_seqs, N, B, d_E, d_C, stream);
-        case 3: return launch_energy_w<6>(d_seqs, N, B, d_E, d_C, stream);
+    switch ((N + 31) / 32) {
+        case 1: return launch_energy_w<1>(d_seqs, N, B, d_E, d_C, stream);
+        case 2: return launch_energy_w<2>(d_seqs, N, B, d_E, d_C, stream);
+        case 3: return launch_energy_w<3>(d_seqs, N, B, d_E, d_C, stream);
+        case 4: return launch_energy_w<4>(d_seqs, N, B, d_E, d_C, stream);
+        case 5: return launch_energy_w<5>(d_seqs, N, B, d_E, d_C, stream);
+        case 6: return launch_energy_w<6>(d_seqs, N, B, d_E, d_C, stream);
+        case 7: return launch_energy_w<7>(d_seqs, N, B, d_E, d_C, stream);
         default: return launch_energy_w<8>(d_seqs, N, B, d_E, d_C, stream);
     }
 }

@@ -59,24 +59,85 @@ __device__ __forceinline__ int32_t warp_energy(const uint32_t (&B)[NW], int N, i
     return __reduce_add_sync(kFull, sq);
 }
 
-// Energy of one sequence computed by a single thread (bits in `w`).
-template <int NW>
+// sum_i popc(w[i]) * weight with as few popcounts as full adders (two LOP3
+// each) leave: a popcount takes the XU pipe 8 cycles a warp, a logic
+// instruction the ALU pipe 2, so an adder that saves a popcount is worth it
+// where popcounts fill their pipe.
+template <int n, int weight = 1>
+__device__ __forceinline__ int popc_words(const uint32_t (&w)[n]) {
+    if constexpr (n <= 2) {
+        int s = 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) s += __popc(w[i]);
+        return s * weight;
+    } else {
+        constexpr int f = (n - 1) / 2;
+        uint32_t carry[f];
+        uint32_t acc = w[0];
+#pragma unroll
+        for (int i = 0; i < f; ++i) {
+            const uint32_t a = acc, b = w[1 + 2 * i], c = w[2 + 2 * i];
+            acc = a ^ b ^ c;
+            carry[i] = (a & b) | (c & (a | b));
+        }
+        int s = __popc(acc);
+        if constexpr (n - 2 * f == 2) s += __popc(w[n - 1]);
+        return s * weight + popc_words<f, 2 * weight>(carry);
+    }
+}
+
+// Pairs (i, i + l + 32q) of B with unequal bits: `mask[x]` holds the bits of
+// word x below N - l, so the pairs end where i + l + 32q does.  The masks are
+// those of the last words only, whatever q.
+template <int NW, int q>
+__device__ __forceinline__ int unequal_pairs(const uint32_t (&B)[NW], const uint32_t (&mask)[NW], int l) {
+    uint32_t x[NW - q];
+#pragma unroll
+    for (int w = 0; w + q < NW; ++w)
+        x[w] = (B[w] ^ __funnelshift_r(B[w + q], w + q + 1 < NW ? B[w + q + 1] : 0u, l)) & mask[w + q];
+    return popc_words<NW - q>(x);
+}
+
+// mask[x] = bits of word x below N - l.  TIGHT: N > 32 (NW - 1), and only the
+// last two words can end inside.
+template <int NW, bool TIGHT>
+__device__ __forceinline__ void pair_masks(int N, int l, uint32_t (&mask)[NW]) {
+#pragma unroll
+    for (int x = 0; x < NW; ++x) mask[x] = TIGHT && x + 2 < NW ? kFull : word_lowmask(x, N - l);
+}
+
+template <int NW, bool TIGHT, int q = 0>
+__device__ __forceinline__ int32_t sum_squares(const uint32_t (&B)[NW], const uint32_t (&mask)[NW], int N, int l) {
+    if constexpr (q == NW) {
+        return 0;
+    } else {
+        const int32_t pairs = N - l - 32 * q;  // below 1 only past the last C_k
+        const int32_t Ck = (q + 1 < NW && TIGHT ? pairs : max(pairs, 0)) - 2 * unequal_pairs<NW, q>(B, mask, l);
+        return Ck * Ck + sum_squares<NW, TIGHT, q + 1>(B, mask, N, l);
+    }
+}
+
+// Energy of one sequence computed by a single thread (bits in `B`).
+template <int NW, bool TIGHT = false>
 __device__ __forceinline__ int32_t thread_energy(const uint32_t (&B)[NW], int N) {
-    int32_t E = 0;
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
+    int32_t E = -N * N;  // k = 0 is summed below
+    if constexpr (TIGHT && NW >= 2) {
+        // the masks of the last two words as one 64-bit mask, a bit shorter each round
+        uint32_t mask[NW];
+        pair_masks<NW, true>(N, 0, mask);
+        uint64_t last = (static_cast<uint64_t>(mask[NW - 1]) << 32) | mask[NW - 2];
+#pragma unroll 2
         for (int l = 0; l < 32; ++l) {
-            const int k = 32 * q + l;
-            if (k < 1 || k > N - 1) continue;
-            int cnt = 0;
-#pragma unroll
-            for (int w = 0; w + q < NW; ++w) {
-                const uint32_t xk =
-                    __funnelshift_r(B[w + q], (w + q + 1 < NW) ? B[w + q + 1] : 0u, l);
-                cnt += __popc((B[w] ^ xk) & word_lowmask(w, N - k));
-            }
-            const int32_t Ck = (N - k) - 2 * cnt;
-            E += Ck * Ck;
+            mask[NW - 2] = static_cast<uint32_t>(last);
+            mask[NW - 1] = static_cast<uint32_t>(last >> 32);
+            E += sum_squares<NW, true>(B, mask, N, l);
+            last >>= 1;
+        }
+    } else {
+        for (int l = 0; l < 32; ++l) {
+            uint32_t mask[NW];
+            pair_masks<NW, TIGHT>(N, l, mask);
+            E += sum_squares<NW, TIGHT>(B, mask, N, l);
         }
     }
     return E;

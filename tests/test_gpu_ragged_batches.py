@@ -45,3 +45,26 @@ def test_skew_deviation(labs, orc, N, B):
     clean = sequences(N, B, dirty=False)
     for b in range(B):
         assert got[b] == orc.skew_deviation(clean[b], N)
+
+
+@pytest.mark.parametrize("N", NS)
+def test_energies_and_correlations(labs, orc, N):
+    """Each way a batch is split: a warp a sequence one by one, four by four, a thread a
+    sequence; the rows past the first few repeat them, so the oracle is asked once."""
+    few = 37
+    a = sequences(N, few, dirty=True)
+    clean = sequences(N, few, dirty=False)
+    ora = [orc.energy(x, N, with_C=True) for x in clean]
+    E0 = np.array([e for e, _ in ora], dtype=np.int32)
+    C0 = np.array([c for _, c in ora], dtype=np.int32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nw = (N + 31) // 32
+    for B in (1, few, 32 * sms, 32 * sms + 1, 8 * nw * nw * sms, 8 * nw * nw * sms + 3):
+        rep = -(-B // few)
+        d = dev(np.tile(a, (rep, 1))[:B])
+        want = np.tile(E0, rep)[:B]
+        assert np.array_equal(labs.energy_batch(d, N).cpu().numpy(), want)
+        if B <= 32 * sms + 1:
+            E, C = labs.energy_batch(d, N, with_C=True)
+            assert np.array_equal(E.cpu().numpy(), want)
+            assert np.array_equal(C.cpu().numpy(), np.tile(C0, (rep, 1))[:B])
