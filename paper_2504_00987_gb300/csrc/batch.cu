@@ -92,9 +92,10 @@ __device__ __forceinline__ void batch_unit(const BatchArgs& a, unsigned char* ba
     }
 }
 
-// Pairs take as many registers as they need (see serve_quantum_kernel).
+// Pairs and eight words take as many registers as they need, the others 128
+// (see kMinBlocks).
 template <int NWMAX, int WPS>
-__global__ void __launch_bounds__(256, WPS == 2 ? 1 : 0) batch_kernel(const BatchArgs a) {
+__global__ void __launch_bounds__(256, WPS == 2 || NWMAX > 6 ? 1 : 2) batch_kernel(const BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PairLink links[WPS == 2 ? 4 : 1];  // one per pair of an 8-warp CTA
     const int lane = threadIdx.x & 31;

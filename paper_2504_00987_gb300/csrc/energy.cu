@@ -50,16 +50,6 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_thread_kernel(const uin
     E[b] = thread_energy<NW, true>(s, N);
 }
 
-// C_k of the lane's k = lane + 32q.
-template <int NW, int q = 0>
-__device__ __forceinline__ void lane_correlations(const uint32_t (&s)[NW], const uint32_t (&mask)[NW], int N, int lane,
-                                                  int32_t (&c)[NW]) {
-    if constexpr (q < NW) {
-        c[q] = max(N - lane - 32 * q, 0) - 2 * unequal_pairs<NW, q>(s, mask, lane);
-        lane_correlations<NW, q + 1>(s, mask, N, lane, c);
-    }
-}
-
 // A warp takes ROWS consecutive sequences at a time, so that one's loads and
 // reduction overlap the others' work.
 template <int NW, int ROWS>

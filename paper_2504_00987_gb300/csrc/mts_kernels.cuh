@@ -17,8 +17,16 @@
 
 namespace lgpu {
 
+// Four CTAs per SM (one warp each on a sub-partition) leave 128 registers a
+// thread.  Without a bound the compiler aims at more CTAs than the workloads
+// put on an SM and squeezes the step (N = 64 64 registers, 217 cycles a step
+// for a lone warp against 204; N = 120 96, 359 against 330).  Eight words need
+// more (four CTAs: 556 cycles at N = 256, two: 502).
+template <int NW>
+constexpr int kMinBlocks = NW <= 6 ? 4 : 2;
+
 template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) mts_kernel(const MtsArgs a) {
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_kernel(const MtsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -53,7 +61,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) mts_kernel(const MtsArgs 
 // record of another run (N, K, variant, seed or instance) is left untouched
 // and the replica reports LABS_RUN_BADSTATE.
 template <int NW, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) mts_resume_kernel(const ResumeArgs ra) {
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_resume_kernel(const ResumeArgs ra) {
     extern __shared__ __align__(16) unsigned char smem[];
     const MtsArgs& a = ra.m;
     const int lane = threadIdx.x & 31;
@@ -137,7 +145,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) mts_resume_kernel(const R
 }
 
 template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) tabu_kernel(const TabuArgs a) {
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) tabu_kernel(const TabuArgs a) {
     __shared__ __align__(16) int32_t Cs_all[kWarpsPerBlock][kTabuScratchInts<NW>];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;

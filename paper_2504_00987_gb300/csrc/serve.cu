@@ -128,10 +128,11 @@ __device__ void serve_slot(const ServeArgs& a, int i, int slot, const labs_insta
     }
 }
 
-// Pairs take as many registers as they need (at most one CTA per SM is
-// promised, which spares them spills); single warps keep the default budget.
+// Pairs and eight words take as many registers as they need (at most one CTA
+// per SM is promised, which spares them spills); the others take 128, as the
+// replica kernels do (kMinBlocks).
 template <int NW, int WPS>
-__global__ void __launch_bounds__(256, WPS == 2 ? 1 : 0) serve_quantum_kernel(const ServeArgs a) {
+__global__ void __launch_bounds__(256, WPS == 2 || NW > 6 ? 1 : 2) serve_quantum_kernel(const ServeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PairLink links[WPS == 2 ? 4 : 1];  // one per pair of an 8-warp CTA
     const int lane = threadIdx.x & 31;

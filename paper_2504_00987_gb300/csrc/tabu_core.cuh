@@ -4,18 +4,11 @@
 // delta_k(j) = -2 s_j (s_{j+k} + s_{j-k}) (terms outside 1..N dropped), so
 //   E_j = E + sum_k delta_k (2 C_k + delta_k)
 //       = E + 4(N-1) + 8 M_j - 4 s_j R_j,
-// with M_j = sum_{k>=1} s_{j+k} s_{j-k} (a masked popcount of the XOR of the
-// two windows of j) and R_j = sum_k C_k (s_{j+k} + s_{j-k}).  R_j is set up
-// once per search on bit planes (0-based bits b_i, s_i = 2 b_i - 1):
-//   R_j = 2 S_j - T_j,  S_j = sum_k C_k (b_{j+k} + b_{j-k}),
-//   T_j = sum_{k<=j} C_k + sum_{k<=N-1-j} C_k,
-// where S_j = sum_m w_m [popc(t_m & X_j) + popc(t_m & Y_j)] over the
-// two's-complement planes t_m of C_k (from warp ballots), X_j = pivot >> j
-// (bit k = b_{j+k}) and Y_j the mirrored window (bit k = b_{j-k}); T_j comes
-// from prefix sums of C_k.  After every move each neighbour's energy change
-// is updated exactly in O(1) from C_k and the self-convolution V_m of the
-// spins (the identity stands above tabu_search), so a step never goes back to
-// the bits.  Arithmetic is exact int32.
+// with M_j = sum_{k>=1} s_{j+k} s_{j-k} and R_j = sum_k C_k (s_{j+k} + s_{j-k}),
+// which search_setup computes once per search.  After every move each
+// neighbour's energy change is updated exactly in O(1) from C_k and the
+// self-convolution V_m of the spins (the identity stands above tabu_search),
+// so a step never goes back to the bits.  Arithmetic is exact int32.
 //
 // Work split: lane l owns the neighbours j = l + 32q: their keys (energy
 // change, index and spin in one int), tabu expiry and spins in registers; V,
@@ -25,38 +18,19 @@
 #pragma once
 
 #include <climits>
+#include <type_traits>
 
 #include "labs_device.cuh"
 
 namespace lgpu {
 
-// C_k = (N - k) - 2 popc(b_i xor b_{i+k} over i < N-k) for the lane's
-// k = lane + 32q (C_0 and C_{k >= N} are 0).
-template <int NW>
-__device__ __forceinline__ void correlations(const uint32_t (&B)[NW], int N, int lane,
-                                             int32_t (&c)[NW]) {
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-        const int k = lane + 32 * q;
-        int cnt = 0;
-#pragma unroll
-        for (int w = 0; w + q < NW; ++w) {
-            const uint32_t xk = __funnelshift_r(B[w + q], (w + q + 1 < NW) ? B[w + q + 1] : 0u, lane);
-            cnt += __popc((B[w] ^ xk) & word_lowmask(w, N - k));
-        }
-        c[q] = (k >= 1 && k <= N - 1) ? (N - k) - 2 * cnt : 0;
+// f(integral_constant<int, 0>) .. f(integral_constant<int, n - 1>).
+template <int n, int i = 0, class F>
+__device__ __forceinline__ void for_each_index(F&& f) {
+    if constexpr (i < n) {
+        f(std::integral_constant<int, i>{});
+        for_each_index<n, i + 1>(f);
     }
-}
-
-// Energy of the warp-uniform sequence B (all lanes return it).
-template <int NW>
-__device__ __forceinline__ int32_t warp_energy(const uint32_t (&B)[NW], int N, int lane) {
-    int32_t c[NW];
-    correlations<NW>(B, N, lane, c);
-    int32_t sq = 0;
-#pragma unroll
-    for (int q = 0; q < NW; ++q) sq += c[q] * c[q];
-    return __reduce_add_sync(kFull, sq);
 }
 
 // sum_i popc(w[i]) * weight with as few popcounts as full adders (two LOP3
@@ -104,6 +78,16 @@ template <int NW, bool TIGHT>
 __device__ __forceinline__ void pair_masks(int N, int l, uint32_t (&mask)[NW]) {
 #pragma unroll
     for (int x = 0; x < NW; ++x) mask[x] = TIGHT && x + 2 < NW ? kFull : word_lowmask(x, N - l);
+}
+
+// C_k of the lane's k = lane + 32q (C_0 = N, C_{k >= N} = 0); `mask` as for l = lane.
+template <int NW, int q = 0>
+__device__ __forceinline__ void lane_correlations(const uint32_t (&s)[NW], const uint32_t (&mask)[NW], int N, int lane,
+                                                  int32_t (&c)[NW]) {
+    if constexpr (q < NW) {
+        c[q] = max(N - lane - 32 * q, 0) - 2 * unequal_pairs<NW, q>(s, mask, lane);
+        lane_correlations<NW, q + 1>(s, mask, N, lane, c);
+    }
 }
 
 template <int NW, bool TIGHT, int q = 0>
@@ -188,201 +172,30 @@ __device__ __forceinline__ bool pair_exchange(PairLink* link, int half, uint32_t
     return ok;
 }
 
-// Bit-plane count bound: |C_k| <= N - 1 < 32*NW, so C_k fits in
-// bitlen(32*NW - 1) + 1 two's-complement bits.
-template <int NW>
-struct PlaneMax {
-    static constexpr int value = (NW == 2) ? 7 : (NW <= 4) ? 8 : 9;
-};
-
-// sum_i popc(w[i]) * weight for n words, carry-save compressed: full
-// adders (sum = a^b^c, carry = maj(a,b,c), one LOP3 each) fold three words
-// of one weight into one word of that weight and one of twice the weight,
-// so n words cost about n/2 + log n popcounts instead of n.  The adders
-// trade popcounts (XU pipe) for logic (ALU pipe), which pays while the
-// step has registers to spare: for 7 or more words (six- and eight-word
-// sequences, N > 160) plain popcounts measured 14-21 % faster on GB300
-// and 2-16 % slower below; five-word sequences (6 words) count plainly as
-// well.  Five words (four-word sequences) take one full adder and two plain
-// popcounts, about 1 % faster than two adders.
-template <int n, int weight>
-__device__ __forceinline__ int csa_popc(const uint32_t (&w)[n]) {
-    if constexpr (weight == 1 && n == 5) {
-        const uint32_t a = w[0], b = w[1], c = w[2];
-        return __popc(a ^ b ^ c) + 2 * __popc((a & b) | (c & (a | b))) + __popc(w[3]) + __popc(w[4]);
-    } else if constexpr (n <= 2 || (weight == 1 && n >= 6)) {
-        int s = 0;
-#pragma unroll
-        for (int i = 0; i < n; ++i) s += __popc(w[i]);
-        return s * weight;
-    } else {
-        constexpr int f = (n - 1) / 2;  // full adders at this weight
-        uint32_t carry[f];
-        uint32_t acc = w[0];
-#pragma unroll
-        for (int i = 0; i < f; ++i) {
-            const uint32_t a = acc, b = w[1 + 2 * i], c = w[2 + 2 * i];
-            acc = a ^ b ^ c;
-            carry[i] = (a & b) | (c & (a | b));
-        }
-        int s = __popc(acc);
-        if constexpr (n - 2 * f == 2) s += __popc(w[n - 1]);
-        return s * weight + csa_popc<f, 2 * weight>(carry);
-    }
-}
-
-// S[q] += sum over planes m < P of w_m [popc(t_m & X_q) + popc(t_m & Y_q)],
-// plane 0 being the constant parity pattern of C_k (C_k = N - k mod 2) and
-// plane P-1 the sign plane (weight -2^(P-1)).  Fully unrolled for a
-// compile-time P so every ballot and popcount of the step can overlap.
-template <int NW, int P>
-__device__ __forceinline__ void score_planes(const int32_t (&c)[NW], const uint32_t (&par)[NW],
-                                             const uint32_t (&X)[NW][NW],
-                                             const uint32_t (&Y)[NW][NW], int32_t (&S)[NW]) {
-#pragma unroll
-    for (int m = 0; m < P; ++m) {
-        uint32_t tp[NW];
-#pragma unroll
-        for (int w = 0; w < NW; ++w) tp[w] = (m == 0) ? par[w] : __ballot_sync(kFull, (c[w] >> m) & 1);
-        constexpr int32_t one = 1;
-        const int32_t wm = (m == P - 1) ? -(one << m) : (one << m);
-#pragma unroll
-        for (int q = 0; q < NW; ++q) {
-            uint32_t words[NW + 1];  // (NW - q) words of X_j and (q + 1) of Y_j
-#pragma unroll
-            for (int w = 0; w + q < NW; ++w) words[w] = tp[w] & X[q][w];
-#pragma unroll
-            for (int w = 0; w <= q; ++w) words[NW - q + w] = tp[w] & Y[q][w];
-            S[q] += csa_popc<NW + 1, 1>(words) * wm;
-        }
-    }
-}
-
-// Inclusive prefix sums of C at the lane's own indices: pc[q] = PC(l + 32q),
-// PC(n) = sum_{k=1}^{n} C_k (C_0 = 0).  Two chunks share one packed 32-bit
-// shuffle scan (low and high 16-bit halves; every within-chunk prefix is
-// bounded by 32 (N-1) < 2^15).  Used once per search; afterwards the sums
-// are updated incrementally per move.
-template <int NW>
-__device__ __forceinline__ void prefix_own(const int32_t (&c)[NW], int lane, int32_t (&pc)[NW]) {
-    constexpr int NP = NW & ~1;  // chunks scanned in pairs
-    int32_t carry = 0;
-#pragma unroll
-    for (int q = 0; q < NP; q += 2) {
-        int32_t v = c[q] + c[q + 1] * 65536;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t n = __shfl_up_sync(kFull, v, o);
-            if (lane >= o) v += n;
-        }
-        const int32_t last = __shfl_sync(kFull, v, 31);
-        const int32_t lo = static_cast<int32_t>(static_cast<int16_t>(v & 0xFFFF));
-        const int32_t hi = (v - lo) / 65536;
-        const int32_t lo31 = static_cast<int32_t>(static_cast<int16_t>(last & 0xFFFF));
-        const int32_t hi31 = (last - lo31) / 65536;
-        pc[q] = carry + lo;
-        pc[q + 1] = carry + lo31 + hi;
-        carry += lo31 + hi31;
-    }
-    if constexpr (NW & 1) {  // an odd word count leaves one chunk, scanned alone
-        int32_t v = c[NW - 1];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t n = __shfl_up_sync(kFull, v, o);
-            if (lane >= o) v += n;
-        }
-        pc[NW - 1] = carry + v;
-    }
-}
-
-// T_j = PC(j) + PC(N-1-j) for the lane's j = l + 32q: its own prefix plus
-// the mirror index's prefix, read back through the warp's shared scratch.
-template <int NW>
-__device__ __forceinline__ void mirror_terms(const int32_t (&pc)[NW], int N, int lane,
-                                             int32_t* __restrict__ Cs, int32_t (&T)[NW]) {
-#pragma unroll
-    for (int q = 0; q < NW; ++q) Cs[lane + 32 * q] = pc[q];
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-        const int j = lane + 32 * q;
-        T[q] = pc[q] + Cs[j < N ? N - 1 - j : 0];
-    }
-    __syncwarp();
-}
-
-// Scores S_j with P bit planes, where P >= the planes C_k needs (extra
-// planes only repeat the sign and leave the sum exact).  Three fully
-// unrolled widths keep the code small enough for the instruction cache
-// (a jump table over every width measured several hundred cycles slower).
-template <int NW>
-__device__ __forceinline__ void score_dispatch(int P, const int32_t (&c)[NW], const uint32_t (&par)[NW],
-                                               const uint32_t (&X)[NW][NW], const uint32_t (&Y)[NW][NW],
-                                               int32_t (&S)[NW]) {
-#pragma unroll
-    for (int q = 0; q < NW; ++q) S[q] = 0;
-    if (P <= 5)
-        score_planes<NW, 5>(c, par, X, Y, S);
-    else if (P <= 6)
-        score_planes<NW, 6>(c, par, X, Y, S);
-    else
-        score_planes<NW, PlaneMax<NW>::value>(c, par, X, Y, S);
-}
-
-// Number of two's-complement planes that hold every C_k of the warp:
-// bit length of max |C_k| plus the sign bit.
-template <int NW>
-__device__ __forceinline__ int plane_count(const int32_t (&c)[NW]) {
-    uint32_t mx = 0;
-#pragma unroll
-    for (int q = 0; q < NW; ++q) mx = max(mx, static_cast<uint32_t>(abs(c[q])));
-    return 33 - __clz(__reduce_max_sync(kFull, mx));
-}
-
-// The lane's windows of an NW-word vector: XB[i] = word i of B >> lane and
-// YB[i] = word i of RL >> (31 - lane).  For j = lane + 32q, word w of the
-// forward window X_j (bit k = b_{j+k}) is XB[q + w] and word w of the
-// backward window Y_j (bit k = b_{j-k}) is YB[w + NW - 1 - q]; both are zero
-// past the ends of the sequence.
-template <int NW>
-__device__ __forceinline__ void pivot_windows(const uint32_t (&B)[NW], const uint32_t (&RL)[NW],
-                                              int lane, uint32_t (&XB)[NW], uint32_t (&YB)[NW]) {
-#pragma unroll
-    for (int i = 0; i < NW; ++i) {
-        XB[i] = __funnelshift_r(B[i], i + 1 < NW ? B[i + 1] : 0u, lane);
-        YB[i] = __funnelshift_r(RL[i], i + 1 < NW ? RL[i + 1] : 0u, 31 - lane);
-    }
-}
-
 // Scratch of one warp's tabu search (ints): V (2 NB), C (2 NB), spins (3 NB
 // bytes), NB = 32 NW; a multiple of 16 bytes.
 template <int NW>
 constexpr int kTabuScratchInts = 128 * NW + 24 * NW;
 
-// V_m = sum_a s_a s_{m-a} (terms outside 0..N-1 dropped) for m = lane + 32i,
-// i < 2 NW, from the bits of the sequence and its mirror image.
-template <int NW>
-__device__ __forceinline__ void store_self_convolution(const uint32_t (&B)[NW], const uint32_t (&RL)[NW], int N,
-                                                       int lane, int32_t* __restrict__ Vs) {
-    // Z[x + 1] = word x of RL >> (31 - lane), x = -1 .. NW-1: bit i of word
-    // w + NW - 1 - i' is b_{m-a} for m = lane + 32 i', a = 32 w + i
-    uint32_t Z[NW + 1];
-    Z[0] = __funnelshift_r(0u, RL[0], 31 - lane);
+// V_m = sum_a x_a x_{m-a} for m = lane + 32i <= N - 1, stored at V[m] (or at
+// V[2N - 2 - m], MIRROR, where X is the sequence reversed): bits X and their
+// full-width reversal XL.  a runs over 0..m, so only the last word is cut.
+template <int NW, bool MIRROR>
+__device__ __forceinline__ void store_self_convolution(const uint32_t (&X)[NW], const uint32_t (&XL)[NW], int N,
+                                                       int lane, int32_t* __restrict__ V) {
+    uint32_t Y[NW];  // word w + NW - 1 - i: bit a of word w is x_{m-a}
 #pragma unroll
-    for (int x = 0; x < NW; ++x) Z[x + 1] = __funnelshift_r(RL[x], x + 1 < NW ? RL[x + 1] : 0u, 31 - lane);
+    for (int x = 0; x < NW; ++x) Y[x] = __funnelshift_r(XL[x], x + 1 < NW ? XL[x + 1] : 0u, 31 - lane);
+    const uint32_t low_l = 0xFFFFFFFFu >> (31 - lane);  // bits 0..lane
+    auto one = [&](auto I) {
+        constexpr int i = decltype(I)::value;
+        uint32_t diff[i + 1];
 #pragma unroll
-    for (int i = 0; i < 2 * NW; ++i) {
+        for (int w = 0; w <= i; ++w) diff[w] = (X[w] ^ Y[w + NW - 1 - i]) & (w == i ? low_l : kFull);
         const int m = lane + 32 * i;
-        const int lo = max(0, m - N + 1), hi = min(m, N - 1);  // a in [lo, hi]
-        int diff = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const int x = w + NW - 1 - i;  // compile-time
-            if (x >= -1 && x < NW)
-                diff += __popc((B[w] ^ Z[x + 1]) & word_lowmask(w, hi + 1) & ~word_lowmask(w, lo));
-        }
-        Vs[m] = max(hi - lo + 1, 0) - 2 * diff;
-    }
+        if (m <= N - 1) V[MIRROR ? 2 * N - 2 - m : m] = m + 1 - 2 * popc_words<i + 1>(diff);
+    };
+    for_each_index<NW>(one);
 }
 
 // The scratch's parts: V_m, m = 0 .. 2 NB - 1; C_d at C[d] and C[-d]; -2 s~_i
@@ -399,54 +212,87 @@ struct TabuScratch {
 // Fills the scratch for a search from `seq` and returns its energy; s[q] is
 // the spin (0 for j >= N) and d4[q] the energy change D_j / 4 of the lane's
 // j = lane + 32q (unset for j >= N).
+//
+// R_j = sum_i s_i C_{|i-j|} are NB^2 products of small integers: four to an
+// instruction as bytes (__dp4a).  The bytes of C, at both signs of the index,
+// stand in V's place until V is made; a lane reads the aligned words around
+// its own offset -lane once, shifts each pair into place once, and uses the
+// result for all its j = lane + 32q, whose windows lie 8 words apart.  C_k
+// fits a byte for N <= 128 and in nearly every longer sequence; where it does
+// not, the high bits (C_k >> 1) and the low bit go one after the other.
 template <int NW>
 __device__ __forceinline__ int32_t search_setup(const uint32_t (&seq)[NW], int N, int lane,
                                                 int32_t* __restrict__ Cs, int32_t (&s)[NW], int32_t (&d4)[NW]) {
     constexpr int NB = 32 * NW;
     const TabuScratch<NW> sh(Cs);
     int32_t c[NW];
-    correlations<NW>(seq, N, lane, c);
+    {
+        uint32_t mask[NW];
+        pair_masks<NW, false>(N, lane, mask);
+        lane_correlations<NW>(seq, mask, N, lane, c);
+    }
+    if (lane == 0) c[0] = 0;
     int32_t sq = 0;
-#pragma unroll
-    for (int q = 0; q < NW; ++q) sq += c[q] * c[q];
-    const int32_t E = __reduce_add_sync(kFull, sq);
-    // R_j = 2 S_j - T_j from the bit planes of C_k (S_j) and the prefix sums
-    // of C_k (T_j = PC(j) + PC(N-1-j))
-    uint32_t RL[NW], XB[NW], YB[NW], par[NW];
-    reverse_bits<NW>(seq, RL);
-    pivot_windows<NW>(seq, RL, lane, XB, YB);
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t alt = ((N - 32 * w) & 1) ? 0x55555555u : 0xAAAAAAAAu;  // (N - k) odd
-        par[w] = alt & word_lowmask(w, N) & (w == 0 ? ~1u : kFull);
-    }
-    uint32_t X[NW][NW], Y[NW][NW];
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-#pragma unroll
-        for (int w = 0; w + q < NW; ++w) X[q][w] = XB[q + w];
-#pragma unroll
-        for (int w = 0; w <= q; ++w) Y[q][w] = YB[w + NW - 1 - q];
-    }
-    int32_t S[NW], pc[NW], T[NW];
-    score_dispatch<NW>(plane_count<NW>(c), c, par, X, Y, S);
-    prefix_own<NW>(c, lane, pc);
-    mirror_terms<NW>(pc, N, lane, Cs, T);
-    store_self_convolution<NW>(seq, RL, N, lane, sh.V);
+    bool large = false;
 #pragma unroll
     for (int q = 0; q < NW; ++q) {
         const int j = lane + 32 * q;
-        s[q] = j < N ? ((XB[q] & 1u) ? 1 : -1) : 0;
+        sq += c[q] * c[q];
+        large = large || abs(c[q]) > 127;
+        s[q] = j < N ? 2 * static_cast<int32_t>((seq[q] >> lane) & 1u) - 1 : 0;
         sh.C[j] = c[q];
         sh.C[-j] = c[q];
         sh.S[j] = static_cast<int8_t>(-2 * s[q]);
         sh.S[j - NB] = 0;
         sh.S[j + NB] = 0;
     }
+    const int32_t E = __reduce_add_sync(kFull, sq);
+    const bool split = NW > 4 && __any_sync(kFull, large);
+    int32_t acc[NW];  // -2 R_j
+#pragma unroll
+    for (int q = 0; q < NW; ++q) acc[q] = 0;
+    int8_t* const G = reinterpret_cast<int8_t*>(sh.V) + NB;  // C_{|x|} as a byte at G[x], -NB < x < NB
+    const int32_t* const Gw = reinterpret_cast<const int32_t*>(G) + ((-lane) >> 2);
+    const int32_t* const Sw = reinterpret_cast<const int32_t*>(sh.S);
+    const int bits = 8 * (-lane & 3);
+#pragma unroll 1
+    for (int part = split ? 1 : 0; part >= 0; --part) {
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const int j = lane + 32 * q;
+            const int8_t byte = static_cast<int8_t>(!split ? c[q] : part ? c[q] >> 1 : c[q] & 1);
+            G[j] = byte;
+            G[-j] = byte;
+            acc[q] *= 2;
+        }
+        __syncwarp();
+        int32_t sw[8 * NW];
+#pragma unroll
+        for (int n = 0; n < 8 * NW; ++n) sw[n] = Sw[n];
+        uint32_t lo = Gw[-8 * (NW - 1)];
+#pragma unroll
+        for (int x = -8 * (NW - 1); x < 8 * NW; ++x) {
+            const uint32_t hi = Gw[x + 1];
+            const int32_t u = static_cast<int32_t>(__funnelshift_r(lo, hi, bits));  // C_{|i-j|}, i = 4 (x + 8q) ..
+            lo = hi;
+#pragma unroll
+            for (int q = 0; q < NW; ++q)
+                if (x + 8 * q >= 0 && x + 8 * q < 8 * NW) acc[q] = __dp4a(sw[x + 8 * q], u, acc[q]);
+        }
+        __syncwarp();
+    }
+    {
+        uint32_t RL[NW], RN[NW], BL[NW];
+        reverse_bits<NW>(seq, RL);
+        store_self_convolution<NW, false>(seq, RL, N, lane, sh.V);
+        shr_uniform<NW>(RL, NB - N, RN);  // bit x = b_{N-1-x}
+        reverse_bits<NW>(RN, BL);
+        store_self_convolution<NW, true>(RN, BL, N, lane, sh.V);
+    }
     __syncwarp();
     // D_j / 4 = N - 1 + 2 M_j - s_j R_j, 2 M_j = V_{2j} - 1
 #pragma unroll
-    for (int q = 0; q < NW; ++q) d4[q] = N - 2 + sh.V[2 * (lane + 32 * q)] - s[q] * (2 * S[q] - T[q]);
+    for (int q = 0; q < NW; ++q) d4[q] = N - 2 + sh.V[2 * (lane + 32 * q)] + s[q] * (acc[q] >> 1);
     __syncwarp();
     return E;
 }
@@ -518,12 +364,12 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     static_assert(WPS == 1 || (WPS == 2 && NW % 2 == 0 && HALF >= 0 && HALF < 2), "warps per sequence");
     constexpr int NB = 32 * NW;
     constexpr int QB = HALF * (NW / WPS), QE = (HALF + 1) * (NW / WPS);  // this warp's q
-    // A drawn tie is scored by a second copy of the scoring code from three
-    // words on, and through the loop of the first where two words make that
-    // copy as long as the rest of the step (cycles a step, one warp alone:
-    // N = 64 232 with the copy, 217 without; N = 120 343 and 355; N = 192 414
-    // and 443).
-    constexpr bool kRecompute = NW <= 4 ? NW > 2 : true;
+    // A drawn tie is scored by a second copy of the scoring code at three and
+    // four words, and through the loop of the first at two, where that copy is
+    // as long as the rest of the step, and from five words on, where it costs
+    // registers (cycles a step, one warp alone, with / without the copy: N = 64
+    // 243 / 217, N = 120 343 / 355, N = 160 375 / 358, N = 256 502 / 475).
+    constexpr bool kRecompute = NW <= 4 && NW > 2;
     constexpr int32_t kLow = 511;  // key bits below the energy change
     constexpr int32_t kNone = INT_MAX & ~kLow;  // no candidate: above every key, low bits those of j = 0
     const TabuScratch<NW> sh(Cs);
