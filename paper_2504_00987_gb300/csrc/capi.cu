@@ -136,13 +136,13 @@ int32_t make_mts_args(const labs_params* P, uint64_t seed, uint64_t first_instan
     if (P == nullptr) return fail(LABS_EINVAL, "params is NULL");
     LABS_TRY(check_run(P->N, P->K, P->replace_policy, P->target_E, P->max_generations, P->max_steps,
                        P->max_iter, first_instance, replicas, "params"));
-    if (replicas > (static_cast<int64_t>(1) << 31) * lgpu::kWarpsPerBlock / 2)
+    if (replicas > (static_cast<int64_t>(1) << 32))
         return fail(LABS_EINVAL, "too many replicas for one launch");
     if (P->trace_cap < 0) return fail(LABS_EINVAL, "trace_cap < 0");
     if (P->d_trace != nullptr) LABS_TRY(check_dev(P->d_trace, 16, "d_trace", false));
     LABS_TRY(check_variant(P->variant, P->N, true, "params"));
     const size_t per_warp = lgpu::mts_smem_per_warp(P->N, P->K);
-    if (per_warp * lgpu::kWarpsPerBlock > 227u * 1024u)
+    if (per_warp > lgpu::kCtaSmem)
         return fail(LABS_EINVAL, "population does not fit in shared memory (N=%d, K=%d)", P->N, P->K);
 
     a->N = P->N;

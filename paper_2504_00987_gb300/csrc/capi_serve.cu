@@ -120,6 +120,7 @@ struct labs_server {
     int64_t cls_cap[kClasses] = {};
     int64_t cls_cap2[kClasses] = {};
     int64_t cls_active[kClasses] = {};
+    int64_t sms = 1;
     int pair_wpb = 2;  // CTA size of the two-warps-per-slot launches
     Arena arena;
 
@@ -353,6 +354,10 @@ void scheduler(labs_server* s) {
             e = cudaMemcpyAsync(s->d_active, s->h_active, sizeof(int32_t) * n, cudaMemcpyHostToDevice, s->stream);
         if (e == cudaSuccess) e = cudaEventRecord(s->ev0, s->stream);
         if (e == cudaSuccess) e = cudaEventRecord(s->ev_fork, s->stream);
+        // Few requests spread over the SMs in smaller CTAs (warps on one SM slow
+        // each other): as many warps a CTA as keep one CTA on every SM.
+        int cta_warps = s->opts.warps_per_block;
+        while (cta_warps > 1 && static_cast<int64_t>(n) * 2 <= static_cast<int64_t>(cta_warps) * s->sms) cta_warps /= 2;
         // one launch per class, each on its own stream, joined back into the main one
         for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
             if (seg_len[c] == 0) continue;
@@ -373,7 +378,7 @@ void scheduler(labs_server* s) {
             e = cudaStreamWaitEvent(s->cls_stream[c], s->ev_fork, 0);
             if (e == cudaSuccess)
                 e = lgpu::launch_serve_quantum(a, kClassNw[c], pair ? 2 : 1,
-                                               pair ? s->pair_wpb : s->opts.warps_per_block, s->cls_stream[c]);
+                                               pair ? s->pair_wpb : cta_warps, s->cls_stream[c]);
             if (e == cudaSuccess) e = cudaEventRecord(s->ev_join[c], s->cls_stream[c]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s->stream, s->ev_join[c], 0);
         }
@@ -465,6 +470,7 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
     }
     s->opts = *o;
     s->opts.warps_per_block = cta;
+    s->sms = sm_count();
     s->pair_wpb = std::max(2, cta);
     cudaGetDevice(&s->device);
     // the arena: hbm_budget_bytes, or room for max_slots requests of (max_N, max_K)

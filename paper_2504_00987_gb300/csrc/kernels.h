@@ -10,8 +10,6 @@
 
 namespace lgpu {
 
-constexpr int kWarpsPerBlock = 4;
-
 // Shared scratch of one warp's tabu search over nw 32-bit words: V and C (64 nw
 // ints each) and the spins (96 nw bytes); see tabu_search.
 constexpr size_t tabu_scratch_bytes(int nw) { return 608u * static_cast<size_t>(nw); }

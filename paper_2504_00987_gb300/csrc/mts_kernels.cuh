@@ -17,23 +17,34 @@
 
 namespace lgpu {
 
-// Four CTAs per SM (one warp each on a sub-partition) leave 128 registers a
-// thread.  Without a bound the compiler aims at more CTAs than the workloads
-// put on an SM and squeezes the step (N = 64 64 registers, 217 cycles a step
-// for a lone warp against 204; N = 120 96, 359 against 330).  Eight words need
-// more (four CTAs: 556 cycles at N = 256, two: 502).
+// One warp per CTA: replicas and searches share nothing, so a CTA's end should
+// free no more than its own slot, and few of them spread over the SMs (a lone
+// search of N = 201 takes 73 us on an SM of its own and 87 us beside three
+// others; 5,000 of them, of uneven length, 331 us instead of 394).
+// Sixteen CTAs per SM leave 128 registers a thread.  Without a bound the
+// compiler aims at more warps than the workloads put on an SM and squeezes
+// the step (N = 64 64 registers, 217 cycles a step for a lone warp against
+// 204; N = 120 96, 359 against 330).
 template <int NW>
-constexpr int kMinBlocks = NW <= 6 ? 4 : 2;
+constexpr int kMinBlocks = 16;
+
+// Grid of n one-warp CTAs (n <= 2^32), and the CTA's index in it.
+inline dim3 warp_grid(int64_t n) {
+    constexpr int64_t row = int64_t{1} << 30;
+    return n <= row ? dim3(static_cast<unsigned>(n)) : dim3(static_cast<unsigned>(row), static_cast<unsigned>((n + row - 1) / row));
+}
+__device__ __forceinline__ int64_t warp_index() {
+    return static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x;
+}
 
 template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_kernel(const MtsArgs a) {
+__global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_kernel(const MtsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kWarpsPerBlock + warp;
+    const int lane = threadIdx.x;
+    const int64_t r = warp_index();
     if (r >= a.replicas) return;
 
-    uint32_t* pop = reinterpret_cast<uint32_t*>(smem + static_cast<size_t>(warp) * a.smem_per_warp);
+    uint32_t* pop = reinterpret_cast<uint32_t*>(smem);
     int32_t* popE = reinterpret_cast<int32_t*>(pop + a.K * NW);
     int32_t* Cs = popE + a.K;
     ReplicaCfg cfg;
@@ -61,15 +72,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_kerne
 // record of another run (N, K, variant, seed or instance) is left untouched
 // and the replica reports LABS_RUN_BADSTATE.
 template <int NW, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_resume_kernel(const ResumeArgs ra) {
+__global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_resume_kernel(const ResumeArgs ra) {
     extern __shared__ __align__(16) unsigned char smem[];
     const MtsArgs& a = ra.m;
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kWarpsPerBlock + warp;
+    const int lane = threadIdx.x;
+    const int64_t r = warp_index();
     if (r >= a.replicas) return;
 
-    uint32_t* pop = reinterpret_cast<uint32_t*>(smem + static_cast<size_t>(warp) * a.smem_per_warp);
+    uint32_t* pop = reinterpret_cast<uint32_t*>(smem);
     int32_t* popE = reinterpret_cast<int32_t*>(pop + a.K * NW);
     int32_t* Cs = popE + a.K;
     ReplicaCfg cfg;
@@ -145,11 +155,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) mts_resum
 }
 
 template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) tabu_kernel(const TabuArgs a) {
-    __shared__ __align__(16) int32_t Cs_all[kWarpsPerBlock][kTabuScratchInts<NW>];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t b = static_cast<int64_t>(blockIdx.x) * kWarpsPerBlock + warp;
+__global__ void __launch_bounds__(32, kMinBlocks<NW>) tabu_kernel(const TabuArgs a) {
+    __shared__ __align__(16) int32_t Cs[kTabuScratchInts<NW>];
+    const int lane = threadIdx.x;
+    const int64_t b = warp_index();
     if (b >= a.B) return;
     const int N = a.N;
     const uint2 key = philox_key(a.seed);
@@ -172,14 +181,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) tabu_kern
     TabuOut to;
     if constexpr (SKEW) {
         to = fix ? tabu_search_skew<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1,
-                                                     Cs_all[warp], trace, a.trace_cap, trace_len, lane)
+                                                     Cs, trace, a.trace_cap, trace_len, lane)
                  : tabu_search_skew<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1,
-                                                      Cs_all[warp], trace, a.trace_cap, trace_len, lane);
+                                                      Cs, trace, a.trace_cap, trace_len, lane);
     } else {
         to = fix ? tabu_search<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1,
-                                                Cs_all[warp], trace, a.trace_cap, trace_len, lane)
+                                                Cs, trace, a.trace_cap, trace_len, lane)
                  : tabu_search<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1,
-                                                 Cs_all[warp], trace, a.trace_cap, trace_len, lane);
+                                                 Cs, trace, a.trace_cap, trace_len, lane);
     }
     if (lane < ROW) {
         uint32_t v = 0;
@@ -195,12 +204,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kMinBlocks<NW>) tabu_kern
 
 template <int NW, bool TRACE, bool SKEW>
 cudaError_t launch_mts_t(const MtsArgs& a, cudaStream_t stream) {
-    const size_t smem = a.smem_per_warp * kWarpsPerBlock;
+    const size_t smem = a.smem_per_warp;
     cudaError_t e = cudaFuncSetAttribute(mts_kernel<NW, TRACE, SKEW>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    const int64_t blocks = (a.replicas + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    mts_kernel<NW, TRACE, SKEW><<<static_cast<unsigned>(blocks), kWarpsPerBlock * 32, smem, stream>>>(a);
+    mts_kernel<NW, TRACE, SKEW><<<warp_grid(a.replicas), 32, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -226,12 +234,11 @@ cudaError_t launch_mts_family(const MtsArgs& a, cudaStream_t stream) {
 
 template <int NW, bool SKEW>
 cudaError_t launch_resume_w(const ResumeArgs& a, cudaStream_t stream) {
-    const size_t smem = a.m.smem_per_warp * kWarpsPerBlock;
+    const size_t smem = a.m.smem_per_warp;
     cudaError_t e = cudaFuncSetAttribute(mts_resume_kernel<NW, SKEW>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    const int64_t blocks = (a.m.replicas + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    mts_resume_kernel<NW, SKEW><<<static_cast<unsigned>(blocks), kWarpsPerBlock * 32, smem, stream>>>(a);
+    mts_resume_kernel<NW, SKEW><<<warp_grid(a.m.replicas), 32, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -249,11 +256,10 @@ cudaError_t launch_resume_family(const ResumeArgs& a, cudaStream_t stream) {
 
 template <int NW, bool SKEW>
 cudaError_t launch_tabu_w(const TabuArgs& a, cudaStream_t stream) {
-    const int64_t blocks = (a.B + kWarpsPerBlock - 1) / kWarpsPerBlock;
     if (a.d_trace)
-        tabu_kernel<NW, true, SKEW><<<static_cast<unsigned>(blocks), kWarpsPerBlock * 32, 0, stream>>>(a);
+        tabu_kernel<NW, true, SKEW><<<warp_grid(a.B), 32, 0, stream>>>(a);
     else
-        tabu_kernel<NW, false, SKEW><<<static_cast<unsigned>(blocks), kWarpsPerBlock * 32, 0, stream>>>(a);
+        tabu_kernel<NW, false, SKEW><<<warp_grid(a.B), 32, 0, stream>>>(a);
     return cudaGetLastError();
 }
 
