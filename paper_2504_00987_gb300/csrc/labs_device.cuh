@@ -63,24 +63,6 @@ __device__ __forceinline__ uint32_t word_lowmask(int v, int n) {
     return hi >= 32 ? kFull : (hi <= 0 ? 0u : ((1u << hi) - 1u));
 }
 
-// Position of the (n+1)-th set bit of x (n < popc(x)), by halving.
-__device__ __forceinline__ int nth_set_bit(uint32_t x, int n) {
-    int pos = 0;
-#pragma unroll
-    for (int width = 16; width >= 1; width >>= 1) {
-        const uint32_t lowbits = x & ((1u << width) - 1u);
-        const int c = __popc(lowbits);
-        if (n >= c) {
-            n -= c;
-            x >>= width;
-            pos += width;
-        } else {
-            x = lowbits;
-        }
-    }
-    return pos;
-}
-
 // out = in >> s for an NW-word vector and a warp-uniform runtime shift
 // 0 <= s < 32*NW: word moves by a log-depth select network, then one funnel
 // shift per word.  No dynamic register indexing.
@@ -101,79 +83,11 @@ __device__ __forceinline__ void shr_uniform(const uint32_t (&in)[NW], int s, uin
     for (int w = 0; w < NW; ++w) out[w] = __funnelshift_r(a[w], w + 1 < NW ? a[w + 1] : 0u, bs);
 }
 
-// oa = a >> s and ob = b >> s for two NW-word vectors and one warp-uniform
-// shift 0 <= s < 32*NW: one select network and one set of funnel shifts
-// shared by both.
-template <int NW>
-__device__ __forceinline__ void shr_uniform2(const uint32_t (&a)[NW], const uint32_t (&b)[NW], int s,
-                                             uint32_t (&oa)[NW], uint32_t (&ob)[NW]) {
-    uint32_t x[NW], y[NW];
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        x[w] = a[w];
-        y[w] = b[w];
-    }
-    const int ws = s >> 5;
-#pragma unroll
-    for (int step = 1; step < NW; step <<= 1) {
-        const bool take = (ws & step) != 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            x[w] = take ? (w + step < NW ? x[w + step] : 0u) : x[w];
-            y[w] = take ? (w + step < NW ? y[w + step] : 0u) : y[w];
-        }
-    }
-    const int bs = s & 31;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        oa[w] = __funnelshift_r(x[w], w + 1 < NW ? x[w + 1] : 0u, bs);
-        ob[w] = __funnelshift_r(y[w], w + 1 < NW ? y[w + 1] : 0u, bs);
-    }
-}
-
-// Two-word vectors: one 64-bit shift each (7.6 % less time per 1,024 x 10^5
-// launch at N = 64 on GB300 than the select network, 4 % fewer instructions).
-template <>
-__device__ __forceinline__ void shr_uniform2<2>(const uint32_t (&a)[2], const uint32_t (&b)[2], int s,
-                                                uint32_t (&oa)[2], uint32_t (&ob)[2]) {
-    const uint64_t ra = ((static_cast<uint64_t>(a[1]) << 32) | a[0]) >> s;
-    const uint64_t rb = ((static_cast<uint64_t>(b[1]) << 32) | b[0]) >> s;
-    oa[0] = static_cast<uint32_t>(ra);
-    oa[1] = static_cast<uint32_t>(ra >> 32);
-    ob[0] = static_cast<uint32_t>(rb);
-    ob[1] = static_cast<uint32_t>(rb >> 32);
-}
-
-// Flip bit i (warp-uniform) of an NW-word vector.
-template <int NW>
-__device__ __forceinline__ void flip_bit(uint32_t (&v)[NW], int i) {
-    if constexpr (NW == 2) {  // one 64-bit one-hot mask
-        const uint64_t m = 1ull << i;
-        v[0] ^= static_cast<uint32_t>(m);
-        v[1] ^= static_cast<uint32_t>(m >> 32);
-    } else {
-        const int wi = i >> 5;
-        const uint32_t m = 1u << (i & 31);
-#pragma unroll
-        for (int w = 0; w < NW; ++w) v[w] ^= (w == wi) ? m : 0u;
-    }
-}
-
 // Full-width reversal: bit (32*NW - 1 - i) of out = bit i of in.
 template <int NW>
 __device__ __forceinline__ void reverse_bits(const uint32_t (&in)[NW], uint32_t (&out)[NW]) {
 #pragma unroll
     for (int w = 0; w < NW; ++w) out[w] = __brev(in[NW - 1 - w]);
-}
-
-// Bit i of an NW-word vector (0 <= i < 32*NW; i may differ between lanes).
-template <int NW>
-__device__ __forceinline__ uint32_t get_bit(const uint32_t (&v)[NW], int i) {
-    const int wi = i >> 5;
-    uint32_t x = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) x = (w == wi) ? v[w] : x;
-    return (x >> (i & 31)) & 1u;
 }
 
 // Skew-symmetric completion of an odd-length sequence (Sec. II.C): with

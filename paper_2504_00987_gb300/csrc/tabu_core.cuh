@@ -402,6 +402,7 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     const int32_t* const Cl = C0 + lane;
     const int8_t* const Al = S0 + 2 * lane;
     const int8_t* const Bl = S0 - lane;
+    const uint32_t low_lanes = (1u << lane) - 1u;
 
     while (t < nsteps && !fault && !stuck) {
         // draws of steps t+1 .. t+32, one per lane: tie pick, and expiry of the move's tabu
@@ -491,45 +492,38 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
                         stuck = true;
                         break;
                     }
-                    uint32_t tb[NW];
-    #pragma unroll
+                    int rank[NW];  // minimisers of this warp before the lane's own, in ascending j
+                    int below = 0;
+#pragma unroll
                     for (int q = QB; q < QE; ++q) {
-                        tb[q] = __ballot_sync(kFull, cand[q] <= (kmin | kLow));
-                        if constexpr (WPS == 1) count += __popc(tb[q]);
+                        const uint32_t tb = __ballot_sync(kFull, cand[q] <= (kmin | kLow));
+                        rank[q] = below + __popc(tb & low_lanes);
+                        below += __popc(tb);
                     }
+                    if constexpr (WPS == 1) count = below;
                     const uint32_t u_tie = __shfl_sync(kFull, u_tie_l, t);
                     int idx = static_cast<int>((static_cast<uint64_t>(u_tie) * count) >> 32);
                     if (idx > 0) {  // the idx-th minimiser in ascending j
-                        int p = 0;
                         bool mine = true;  // WPS = 2: the warp holding it finds it, then tells the other
                         if constexpr (WPS == 2) {
                             mine = HALF == 0 ? idx < count_lo : idx >= count_lo;
                             if (HALF == 1) idx -= count_lo;
                         }
-                        if (mine) {
-                            bool found = false;
-    #pragma unroll
-                            for (int q = QB; q < QE; ++q) {
-                                const int pc_q = __popc(tb[q]);
-                                if (!found) {
-                                    if (idx < pc_q) {
-                                        p = 32 * q + nth_set_bit(tb[q], idx);
-                                        found = true;
-                                    } else {
-                                        idx -= pc_q;
-                                    }
-                                }
-                            }
+                        if (mine) {  // its key tells its index and spin
+                            int32_t pick = kNone;
+#pragma unroll
+                            for (int q = QB; q < QE; ++q)
+                                if (cand[q] <= (kmin | kLow) && rank[q] == idx) pick = cand[q];
+                            klow = __reduce_min_sync(kFull, pick) & kLow;
                         }
                         if constexpr (WPS == 2) {
                             uint64_t o = 0;
-                            if (!pair_exchange(link, HALF, (*xseq)++, mine ? static_cast<uint64_t>(p) : 0u, o, lane)) {
+                            if (!pair_exchange(link, HALF, (*xseq)++, mine ? static_cast<uint64_t>(klow) : 0u, o, lane)) {
                                 fault = true;
                                 break;
                             }
-                            if (!mine) p = static_cast<int>(o);
+                            if (!mine) klow = static_cast<int>(o);
                         }
-                        klow = 2 * p + (S0[p] < 0 ? 1 : 0);
                         if constexpr (kRecompute)
                             score_move(klow);
                         else

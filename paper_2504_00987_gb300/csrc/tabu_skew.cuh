@@ -76,6 +76,7 @@ __device__ TabuOut tabu_search_skew(uint32_t (&seq)[NW], const int N, const uint
     const int min_t = max_iter / 10;
     const int max_t = (12 * max_iter) / 100;
     const int nsteps = static_cast<int>(budget < 0 ? max_iter : (budget < max_iter ? budget : max_iter));
+    const uint32_t low_lanes = (1u << lane) - 1u;
     int32_t thr = 0;  // a key below this is a move to below E_best
     int t = 0;        // moves made; this step is t + 1
     bool stuck = false;
@@ -141,31 +142,22 @@ __device__ TabuOut tabu_search_skew(uint32_t (&seq)[NW], const int N, const uint
                     stuck = true;
                     break;
                 }
-                uint32_t tb[NH];
+                int rank[NH];  // minimisers before the lane's own, in ascending i
                 int count = 0;
 #pragma unroll
                 for (int q = 0; q < NH; ++q) {
-                    tb[q] = __ballot_sync(kFull, cand[q] <= (kmin | kLow));
-                    count += __popc(tb[q]);
+                    const uint32_t tb = __ballot_sync(kFull, cand[q] <= (kmin | kLow));
+                    rank[q] = count + __popc(tb & low_lanes);
+                    count += __popc(tb);
                 }
                 const uint32_t u_tie = __shfl_sync(kFull, u_tie_l, t);
-                int idx = static_cast<int>((static_cast<uint64_t>(u_tie) * count) >> 32);
-                if (idx > 0) {  // the idx-th minimiser in ascending i
-                    int p = 0;
-                    bool found = false;
+                const int idx = static_cast<int>((static_cast<uint64_t>(u_tie) * count) >> 32);
+                if (idx > 0) {  // the idx-th minimiser in ascending i: its key tells its index and spin
+                    int32_t pick = kNone;
 #pragma unroll
-                    for (int q = 0; q < NH; ++q) {
-                        const int pc_q = __popc(tb[q]);
-                        if (!found) {
-                            if (idx < pc_q) {
-                                p = 32 * q + nth_set_bit(tb[q], idx);
-                                found = true;
-                            } else {
-                                idx -= pc_q;
-                            }
-                        }
-                    }
-                    klow = 2 * p + (sh.S[p] < 0 ? 1 : 0);
+                    for (int q = 0; q < NH; ++q)
+                        if (cand[q] <= (kmin | kLow) && rank[q] == idx) pick = cand[q];
+                    klow = __reduce_min_sync(kFull, pick) & kLow;
                 }
             }
             // ---- apply: flip b_p and its partner, tenure, bestSeqTS
