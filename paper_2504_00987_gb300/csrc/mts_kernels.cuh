@@ -178,16 +178,17 @@ __global__ void __launch_bounds__(32, kMinBlocks<NW>) tabu_kernel(const TabuArgs
     int4* trace = a.d_trace ? a.d_trace + b * a.trace_cap : nullptr;
     int64_t trace_len = 0;
     const bool fix = (a.variant & LABS_VARIANT_FIX_FIRST_SPIN) != 0;
+    const uint2 draws = step_draws(key, inst, a.generation, 1 + lane);
     TabuOut to;
     if constexpr (SKEW) {
-        to = fix ? tabu_search_skew<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1,
+        to = fix ? tabu_search_skew<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1, draws,
                                                      Cs, trace, a.trace_cap, trace_len, lane)
-                 : tabu_search_skew<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1,
+                 : tabu_search_skew<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1, draws,
                                                       Cs, trace, a.trace_cap, trace_len, lane);
     } else {
-        to = fix ? tabu_search<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1,
+        to = fix ? tabu_search<NW, TRACE, true>(seq, N, key, inst, a.generation, max_iter, -1, draws,
                                                 Cs, trace, a.trace_cap, trace_len, lane)
-                 : tabu_search<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1,
+                 : tabu_search<NW, TRACE, false>(seq, N, key, inst, a.generation, max_iter, -1, draws,
                                                  Cs, trace, a.trace_cap, trace_len, lane);
     }
     if (lane < ROW) {

@@ -30,28 +30,31 @@ struct ReplicaCfg {
     uint2 key;
 };
 
-// Bit j of `mask` is set iff word j%4 of Philox(inst, g, j/4, purpose) < thr
-// (j < N): one Philox block per four bits, nibbles OR-reduced over the warp.
+// Adds the bits of draw block `block` (held by this lane; none if block >= nd)
+// to `mask`: bit j is set iff word j%4 of block j/4 is below thr (j < N).
+// Nibbles are OR-reduced over the warp.
 template <int NW>
-__device__ __forceinline__ void draw_bit_mask(const ReplicaCfg& a, uint32_t g, uint32_t purpose,
-                                              uint32_t thr, int lane, uint32_t (&mask)[NW]) {
+__device__ __forceinline__ void add_draw_bits(const uint4& d, int block, int nd, int N, uint32_t thr,
+                                              uint32_t (&mask)[NW]) {
+    uint32_t nib = (d.x < thr ? 1u : 0u) | (d.y < thr ? 2u : 0u) | (d.z < thr ? 4u : 0u) | (d.w < thr ? 8u : 0u);
+    if (block >= nd) nib = 0u;
+    const int word_of = block >> 3;  // 8 nibbles per 32-bit word
 #pragma unroll
-    for (int w = 0; w < NW; ++w) mask[w] = 0u;
+    for (int w = 0; w < NW; ++w) {
+        const uint32_t part = (word_of == w) ? (nib << (4 * (block & 7))) : 0u;
+        mask[w] |= __reduce_or_sync(kFull, part) & word_lowmask(w, N);
+    }
+}
+
+// Bit j of `mask` is set iff word j%4 of Philox(inst, g, j/4, purpose) < thr
+// (j < N), for the blocks j/4 >= first; `mask` holds the others already.
+template <int NW>
+__device__ __forceinline__ void draw_bit_mask(const ReplicaCfg& a, uint32_t g, uint32_t purpose, uint32_t thr,
+                                              int first, int lane, uint32_t (&mask)[NW]) {
     const int nd = (a.N + 3) / 4;
-    for (int base = 0; base < nd; base += 32) {
-        const int cidx = base + lane;
-        uint32_t nib = 0;
-        if (cidx < nd) {
-            const uint4 d = draw4(a.key, a.inst, g, static_cast<uint32_t>(cidx), purpose);
-            nib = (d.x < thr ? 1u : 0u) | (d.y < thr ? 2u : 0u) | (d.z < thr ? 4u : 0u) |
-                  (d.w < thr ? 8u : 0u);
-        }
-        const int word_of = cidx >> 3;  // 8 nibbles per 32-bit word
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const uint32_t part = (word_of == w) ? (nib << (4 * (cidx & 7))) : 0u;
-            mask[w] |= __reduce_or_sync(kFull, part) & word_lowmask(w, a.N);
-        }
+    for (int base = first; base < nd; base += 32) {
+        const int block = base + lane;
+        add_draw_bits<NW>(draw4(a.key, a.inst, g, static_cast<uint32_t>(block), purpose), block, nd, a.N, thr, mask);
     }
 }
 
@@ -187,21 +190,28 @@ __device__ int64_t replica_generation(const ReplicaCfg& a, ReplicaState<NW>& st,
     const int N = a.N, K = a.K;
     const uint32_t gg = static_cast<uint32_t>(st.g);
     const uint32_t p_mut = a.p_mut_u32;
-    // generation draws: lane 0 -> (g,0), lane 1 -> (g,1), lane 2 -> (g,2)
-    const uint4 gd = draw4(a.key, a.inst, gg, static_cast<uint32_t>(lane < 3 ? lane : 0), kPurposeGen);
-    const uint32_t coin = __shfl_sync(kFull, gd.x, 0);
-    const uint32_t ua = __shfl_sync(kFull, gd.y, 0), ub = __shfl_sync(kFull, gd.z, 0);
-    const uint32_t uc = __shfl_sync(kFull, gd.w, 0), ud = __shfl_sync(kFull, gd.x, 1);
-    const uint32_t ucut = __shfl_sync(kFull, gd.y, 1), usamp = __shfl_sync(kFull, gd.z, 1);
-    const uint32_t uiter = __shfl_sync(kFull, gd.w, 1), urep = __shfl_sync(kFull, gd.x, 2);
+    // One Philox evaluation for the generation's three blocks (lanes 29..31) and
+    // the first 29 mutation blocks, and beside it the one of the first 32 tabu
+    // steps: three evaluations one after the other took 300 cycles more of a
+    // lone warp's generation (N = 64 1,950 around its steps instead of 2,250).
+    constexpr int kMutLanes = 29;
+    const bool gen = lane >= kMutLanes;
+    const uint4 gd = draw4(a.key, a.inst, gg, static_cast<uint32_t>(gen ? lane - kMutLanes : lane),
+                           gen ? kPurposeGen : kPurposeMut);
+    const uint2 draws = step_draws(a.key, a.inst, gg, 1 + lane);
+    const uint32_t coin = __shfl_sync(kFull, gd.x, 29);
+    const uint32_t ua = __shfl_sync(kFull, gd.y, 29), ub = __shfl_sync(kFull, gd.z, 29);
+    const uint32_t uc = __shfl_sync(kFull, gd.w, 29), ud = __shfl_sync(kFull, gd.x, 30);
+    const uint32_t ucut = __shfl_sync(kFull, gd.y, 30), usamp = __shfl_sync(kFull, gd.z, 30);
+    const uint32_t uiter = __shfl_sync(kFull, gd.w, 30), urep = __shfl_sync(kFull, gd.x, 31);
 
     uint32_t child[NW];
     if (coin < a.p_comb_u32) {
         const int p1 = tournament(popE, rand_int(0, K - 1, ua), rand_int(0, K - 1, ub));
         const int p2 = tournament(popE, rand_int(0, K - 1, uc), rand_int(0, K - 1, ud));
         if (a.variant & LABS_VARIANT_UNIFORM_CROSSOVER) {
-            uint32_t m2[NW];  // bits taken from P2
-            draw_bit_mask<NW>(a, gg, kPurposeCross, 0x80000000u, lane, m2);
+            uint32_t m2[NW] = {};  // bits taken from P2
+            draw_bit_mask<NW>(a, gg, kPurposeCross, 0x80000000u, 0, lane, m2);
 #pragma unroll
             for (int w = 0; w < NW; ++w) child[w] = (pop[p1 * NW + w] & ~m2[w]) | (pop[p2 * NW + w] & m2[w]);
         } else {
@@ -217,8 +227,9 @@ __device__ int64_t replica_generation(const ReplicaCfg& a, ReplicaState<NW>& st,
     }
     // Mutate: bit j flips iff word j%4 of (inst, g, j/4, MUT) < p_mut.
     {
-        uint32_t mm[NW];
-        draw_bit_mask<NW>(a, gg, kPurposeMut, p_mut, lane, mm);
+        uint32_t mm[NW] = {};
+        add_draw_bits<NW>(gd, gen ? INT_MAX : lane, (N + 3) / 4, N, p_mut, mm);
+        draw_bit_mask<NW>(a, gg, kPurposeMut, p_mut, kMutLanes, lane, mm);
         if (a.variant & LABS_VARIANT_FIX_FIRST_SPIN) mm[0] &= ~1u;
 #pragma unroll
         for (int w = 0; w < NW; ++w) child[w] ^= mm[w];
@@ -232,15 +243,15 @@ __device__ int64_t replica_generation(const ReplicaCfg& a, ReplicaState<NW>& st,
     TabuOut to;
     if constexpr (SKEW) {
         to = (a.variant & LABS_VARIANT_FIX_FIRST_SPIN)
-                 ? tabu_search_skew<NW, TRACE, true>(child, N, a.key, a.inst, gg, max_iter, budget, Cs,
+                 ? tabu_search_skew<NW, TRACE, true>(child, N, a.key, a.inst, gg, max_iter, budget, draws, Cs,
                                                      trace, trace_cap, trace_len, lane)
-                 : tabu_search_skew<NW, TRACE, false>(child, N, a.key, a.inst, gg, max_iter, budget, Cs,
+                 : tabu_search_skew<NW, TRACE, false>(child, N, a.key, a.inst, gg, max_iter, budget, draws, Cs,
                                                       trace, trace_cap, trace_len, lane);
     } else {
         to = (a.variant & LABS_VARIANT_FIX_FIRST_SPIN)
-                 ? tabu_search<NW, TRACE, true, WPS, HALF>(child, N, a.key, a.inst, gg, max_iter, budget,
+                 ? tabu_search<NW, TRACE, true, WPS, HALF>(child, N, a.key, a.inst, gg, max_iter, budget, draws,
                                                                  Cs, trace, trace_cap, trace_len, lane, link, xseq)
-                 : tabu_search<NW, TRACE, false, WPS, HALF>(child, N, a.key, a.inst, gg, max_iter, budget,
+                 : tabu_search<NW, TRACE, false, WPS, HALF>(child, N, a.key, a.inst, gg, max_iter, budget, draws,
                                                                   Cs, trace, trace_cap, trace_len, lane, link, xseq);
     }
     if (to.fault) {  // the pair lost step: stop the replica, report it

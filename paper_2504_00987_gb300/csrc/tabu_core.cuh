@@ -198,6 +198,12 @@ __device__ __forceinline__ void store_self_convolution(const uint32_t (&X)[NW], 
     for_each_index<NW>(one);
 }
 
+// Tie and tenure draws (x, y) of tabu step t.
+__device__ __forceinline__ uint2 step_draws(uint2 key, uint32_t inst, uint32_t g, int t) {
+    const uint4 r = draw4(key, inst, g, static_cast<uint32_t>(t), kPurposeStep);
+    return make_uint2(r.x, r.y);
+}
+
 // The scratch's parts: V_m, m = 0 .. 2 NB - 1; C_d at C[d] and C[-d]; -2 s~_i
 // at S[i], i = -NB .. 2 NB - 1.
 template <int NW>
@@ -298,7 +304,8 @@ __device__ __forceinline__ int32_t search_setup(const uint32_t (&seq)[NW], int N
 }
 
 // One tabu search from `seq` (warp-uniform).  On return `seq` holds
-// bestSeqTS.  Draws: step t uses Philox(instance, g, t, 4): x tie, y tenure.
+// bestSeqTS.  Draws: step t uses Philox(instance, g, t, 4): x tie, y tenure;
+// `draws` are the lane's of step 1 + lane (step_draws).
 // FIX_FIRST: bit 0 (s_1) is never a candidate move.
 // `Cs` is warp-private shared scratch of kTabuScratchInts<NW> ints.
 // With TRACE, `trace` receives {g, t, j, E} per step while trace_len <
@@ -357,7 +364,7 @@ __device__ __forceinline__ int32_t search_setup(const uint32_t (&seq)[NW], int N
 template <int NW, bool TRACE, bool FIX_FIRST = false, int WPS = 1, int HALF = 0>
 __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key,
                                const uint32_t inst, const uint32_t g, const int max_iter,
-                               const int64_t budget, int32_t* __restrict__ Cs,
+                               const int64_t budget, uint2 draws, int32_t* __restrict__ Cs,
                                int4* __restrict__ trace, const int64_t trace_cap,
                                int64_t& trace_len, const int lane, PairLink* link = nullptr,
                                uint32_t* xseq = nullptr) {
@@ -406,9 +413,9 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
 
     while (t < nsteps && !fault && !stuck) {
         // draws of steps t+1 .. t+32, one per lane: tie pick, and expiry of the move's tabu
-        const uint4 r = draw4(key, inst, g, static_cast<uint32_t>(t + 1 + lane), kPurposeStep);
-        const uint32_t u_tie_l = r.x;
-        const int32_t expiry_l = t + 1 + lane + rand_int(min_t, max_t, r.y);
+        if (t > 0) draws = step_draws(key, inst, g, t + 1 + lane);
+        const uint32_t u_tie_l = draws.x;
+        const int32_t expiry_l = t + 1 + lane + rand_int(min_t, max_t, draws.y);
 #pragma unroll
         for (int q = QB; q < QE; ++q)
             if (K[q] != kNone) K[q] -= off;

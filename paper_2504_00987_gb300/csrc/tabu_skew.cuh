@@ -42,7 +42,7 @@ namespace lgpu {
 template <int NW, bool TRACE, bool FIX_FIRST>
 __device__ TabuOut tabu_search_skew(uint32_t (&seq)[NW], const int N, const uint2 key,
                                     const uint32_t inst, const uint32_t g, const int max_iter,
-                                    const int64_t budget, int32_t* __restrict__ Cs,
+                                    const int64_t budget, uint2 draws, int32_t* __restrict__ Cs,
                                     int4* __restrict__ trace, const int64_t trace_cap,
                                     int64_t& trace_len, const int lane) {
     constexpr int NH = (NW + 1) / 2;  // words of the free half: c < 16 NW
@@ -114,9 +114,9 @@ __device__ TabuOut tabu_search_skew(uint32_t (&seq)[NW], const int N, const uint
 
     while (t < nsteps && !stuck) {
         // draws of steps t+1 .. t+32, one per lane: tie pick, and expiry of the move's tabu
-        const uint4 r = draw4(key, inst, g, static_cast<uint32_t>(t + 1 + lane), kPurposeStep);
-        const uint32_t u_tie_l = r.x;
-        const int32_t expiry_l = t + 1 + lane + rand_int(min_t, max_t, r.y);
+        if (t > 0) draws = step_draws(key, inst, g, t + 1 + lane);
+        const uint32_t u_tie_l = draws.x;
+        const int32_t expiry_l = t + 1 + lane + rand_int(min_t, max_t, draws.y);
         const int tend = min(t + 32, nsteps);
 #pragma unroll 1
         for (; t < tend; ++t) {
