@@ -21,16 +21,16 @@ namespace lgpu {
 
 __device__ __forceinline__ ReplicaCfg serve_cfg(const labs_instance& in) {
     ReplicaCfg c;
-    c.N = in.N;
-    c.K = in.K;
+    c.N = warp_uniform(in.N);
+    c.K = warp_uniform(in.K);
     c.p_comb_u32 = in.p_comb_u32;
     c.p_mut_u32 = in.p_mut_u32;
     c.replace_policy = in.replace_policy;
     c.target_E = in.target_E;
     c.max_generations = in.max_generations;
     c.max_steps = in.max_steps;
-    c.max_iter = in.max_iter;
-    c.variant = in.variant;
+    c.max_iter = warp_uniform(in.max_iter);
+    c.variant = warp_uniform(in.variant);
     c.inst = static_cast<uint32_t>(in.instance);
     c.key = philox_key(in.seed);
     return c;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256, WPS == 2 || NW > 6 ? 1 : 2) serve_quantum
         if (lane < 4) reinterpret_cast<unsigned long long*>(link->slot)[lane] = 0ull;
         __syncthreads();  // every link word is zero before either warp of a pair publishes
     }
-    const int i = (blockIdx.x * (blockDim.x >> 5) + warp) / WPS;
+    const int i = warp_uniform(static_cast<int>(blockIdx.x * (blockDim.x >> 5) + warp) / WPS);
     if (i >= a.n_active) return;
     unsigned char* base = smem + static_cast<size_t>(warp) * a.smem_per_warp;
     const int slot = a.active[i];
