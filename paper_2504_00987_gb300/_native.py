@@ -189,6 +189,8 @@ _lib = None
 def load(path: str = LIB_PATH):
     """Loads liblabs.so; raises if it has not been built (there is no fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
