@@ -369,7 +369,6 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
                                int64_t& trace_len, const int lane, PairLink* link = nullptr,
                                uint32_t* xseq = nullptr) {
     static_assert(WPS == 1 || (WPS == 2 && NW % 2 == 0 && HALF >= 0 && HALF < 2), "warps per sequence");
-    constexpr int NB = 32 * NW;
     constexpr int QB = HALF * (NW / WPS), QE = (HALF + 1) * (NW / WPS);  // this warp's q
     // A drawn tie is scored by a second copy of the scoring code at three and
     // four words, and through the loop of the first at two, where that copy is
@@ -397,10 +396,10 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     const int min_t = max_iter / 10;
     const int max_t = (12 * max_iter) / 100;
     int nsteps = static_cast<int>(budget < 0 ? max_iter : (budget < max_iter ? budget : max_iter));
-    // At two words the loop's bounds as a uniform value take a tenth off a lone
+    // Up to two words the loop's bounds as a uniform value take a tenth off a lone
     // warp's step (N = 64 211 -> 191 cycles); at four words the same hint cost
     // 2.5 % with four warps on a sub-partition.
-    if constexpr (NW == 2) nsteps = warp_uniform(nsteps);
+    if constexpr (NW <= 2) nsteps = warp_uniform(nsteps);
     // Every D_j / 4 loses 4 per move besides the terms below; the keys leave
     // that out, so a stored key is the true one + off, off = 4 << 9 per move
     // since the last multiple of 32.  thr (stored likewise): a key below it is
