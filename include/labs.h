@@ -193,7 +193,9 @@ typedef struct labs_instance {
 
 /* How a batch is mapped on the GPU. */
 typedef struct labs_mapping {
-    int32_t warps_per_block; /* warps per CTA: 1, 2, 4 or 8 */
+    int32_t warps_per_block; /* warps per CTA: 1, 2, 4 or 8 (half as many, in more CTAs,
+                                where their shared memory would not fit one; no result
+                                depends on it) */
     int32_t blocks_per_sm;   /* resident CTAs per SM of the persistent grid, >= 1 */
     int32_t order;           /* LABS_ORDER_* */
     int32_t warps_per_seq;   /* warps per replica: 1 (or 0), or 2 (warps_per_block 2, 4
@@ -398,7 +400,8 @@ typedef struct labs_serve_opts {
     int32_t max_slots;          /* requests resident on the GPU at once (one warp each) */
     int32_t max_N;              /* largest N accepted, 3 .. LABS_MAX_N */
     int32_t max_K;              /* largest K accepted, 1 .. LABS_MAX_K */
-    int32_t warps_per_block;    /* quantum kernel CTA size in warps: 1, 2, 4 or 8 */
+    int32_t warps_per_block;    /* quantum kernel CTA size in warps: 1, 2, 4 or 8; at most, since
+                                   few requests are spread over the SMs in smaller CTAs */
     int64_t quantum_steps;      /* tabu steps per slot per quantum (rounded up to a generation) */
     int64_t queue_capacity;     /* pending requests; submit answers LABS_EBUSY beyond it */
     int64_t hbm_budget_bytes;   /* bytes of the device arena holding the resident

@@ -12,6 +12,7 @@
 
 #include <cuda_runtime.h>
 
+#include "capi_util.h"
 #include "kernels.h"
 #include "replica.cuh"
 
@@ -25,8 +26,17 @@ namespace lgpu {
 // compiler aims at more warps than the workloads put on an SM and squeezes
 // the step (N = 64 64 registers, 217 cycles a step for a lone warp against
 // 204; N = 120 96, 359 against 330).
-template <int NW>
 constexpr int kMinBlocks = 16;
+// Seven and eight words take up to 255 registers while at most eight replicas
+// fall on an SM, which is all those leave room for (128 / 255 registers, one
+// GB300: 152 replicas of N = 256 x 20,000 steps 5.95 / 5.12 ms, 608 of N = 200
+// 5.85 / 4.69, 1,216 of N = 256 8.11 / 7.41); with more, 16 warps on an SM win
+// (a step of 2,432 at N = 256: 1,356 / 1,429 cycles).
+constexpr int kFewBlocks = 8;
+template <int NW>
+inline bool few_replicas(int64_t n) {
+    return NW >= 7 && n <= static_cast<int64_t>(lcapi::sm_count()) * kFewBlocks;
+}
 
 // Grid of n one-warp CTAs (n <= 2^32), and the CTA's index in it.
 inline dim3 warp_grid(int64_t n) {
@@ -37,8 +47,8 @@ __device__ __forceinline__ int64_t warp_index() {
     return static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x;
 }
 
-template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_kernel(const MtsArgs a) {
+template <int NW, bool TRACE, bool SKEW, int BLOCKS>
+__global__ void __launch_bounds__(32, BLOCKS) mts_kernel(const MtsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x;
     const int64_t r = warp_index();
@@ -71,8 +81,8 @@ __global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_kernel(const MtsArgs a
 // from a record at a generation boundary equals the uninterrupted run.  A
 // record of another run (N, K, variant, seed or instance) is left untouched
 // and the replica reports LABS_RUN_BADSTATE.
-template <int NW, bool SKEW>
-__global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_resume_kernel(const ResumeArgs ra) {
+template <int NW, bool SKEW, int BLOCKS>
+__global__ void __launch_bounds__(32, BLOCKS) mts_resume_kernel(const ResumeArgs ra) {
     extern __shared__ __align__(16) unsigned char smem[];
     const MtsArgs& a = ra.m;
     const int lane = threadIdx.x;
@@ -155,7 +165,7 @@ __global__ void __launch_bounds__(32, kMinBlocks<NW>) mts_resume_kernel(const Re
 }
 
 template <int NW, bool TRACE, bool SKEW>
-__global__ void __launch_bounds__(32, kMinBlocks<NW>) tabu_kernel(const TabuArgs a) {
+__global__ void __launch_bounds__(32, kMinBlocks) tabu_kernel(const TabuArgs a) {
     __shared__ __align__(16) int32_t Cs[kTabuScratchInts<NW>];
     const int lane = threadIdx.x;
     const int64_t b = warp_index();
@@ -203,14 +213,21 @@ __global__ void __launch_bounds__(32, kMinBlocks<NW>) tabu_kernel(const TabuArgs
     }
 }
 
-template <int NW, bool TRACE, bool SKEW>
-cudaError_t launch_mts_t(const MtsArgs& a, cudaStream_t stream) {
+template <int NW, bool TRACE, bool SKEW, int BLOCKS>
+cudaError_t launch_mts_b(const MtsArgs& a, cudaStream_t stream) {
     const size_t smem = a.smem_per_warp;
-    cudaError_t e = cudaFuncSetAttribute(mts_kernel<NW, TRACE, SKEW>,
+    cudaError_t e = cudaFuncSetAttribute(mts_kernel<NW, TRACE, SKEW, BLOCKS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    mts_kernel<NW, TRACE, SKEW><<<warp_grid(a.replicas), 32, smem, stream>>>(a);
+    mts_kernel<NW, TRACE, SKEW, BLOCKS><<<warp_grid(a.replicas), 32, smem, stream>>>(a);
     return cudaGetLastError();
+}
+
+template <int NW, bool TRACE, bool SKEW>
+cudaError_t launch_mts_t(const MtsArgs& a, cudaStream_t stream) {
+    if constexpr (NW >= 7 && !TRACE)
+        if (few_replicas<NW>(a.replicas)) return launch_mts_b<NW, TRACE, SKEW, kFewBlocks>(a, stream);
+    return launch_mts_b<NW, TRACE, SKEW, kMinBlocks>(a, stream);
 }
 
 // 32-bit words per sequence in registers.  A step's work grows with them, so
@@ -237,14 +254,21 @@ cudaError_t launch_mts_family(const MtsArgs& a, cudaStream_t stream) {
     }
 }
 
-template <int NW, bool SKEW>
-cudaError_t launch_resume_w(const ResumeArgs& a, cudaStream_t stream) {
+template <int NW, bool SKEW, int BLOCKS>
+cudaError_t launch_resume_b(const ResumeArgs& a, cudaStream_t stream) {
     const size_t smem = a.m.smem_per_warp;
-    cudaError_t e = cudaFuncSetAttribute(mts_resume_kernel<NW, SKEW>,
+    cudaError_t e = cudaFuncSetAttribute(mts_resume_kernel<NW, SKEW, BLOCKS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    mts_resume_kernel<NW, SKEW><<<warp_grid(a.m.replicas), 32, smem, stream>>>(a);
+    mts_resume_kernel<NW, SKEW, BLOCKS><<<warp_grid(a.m.replicas), 32, smem, stream>>>(a);
     return cudaGetLastError();
+}
+
+template <int NW, bool SKEW>
+cudaError_t launch_resume_w(const ResumeArgs& a, cudaStream_t stream) {
+    if constexpr (NW >= 7)
+        if (few_replicas<NW>(a.m.replicas)) return launch_resume_b<NW, SKEW, kFewBlocks>(a, stream);
+    return launch_resume_b<NW, SKEW, kMinBlocks>(a, stream);
 }
 
 template <bool SKEW>

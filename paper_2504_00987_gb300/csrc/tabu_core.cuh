@@ -351,7 +351,9 @@ __device__ __forceinline__ int32_t search_setup(const uint32_t (&seq)[NW], int N
 // of that one vote took 14 cycles more at N = 64 and 37 at N = 120; keeping
 // the best sequence without a branch, 21 and 1 more.
 // Measured, cycles a step, one warp / two / four on an SM sub-partition:
-// N = 64 217 / 295 / 510, N = 120 343 / 453 / 758, N = 192 414 / 574 (two
+// N = 24 174 / 225 / 379, N = 64 191 / 276 / 497, N = 120 331 / 442 / 752,
+// N = 160 366 / 503 / 868; about 23 instructions per 32 neighbours and 60
+// besides, so four warps issue in 80 % of the cycles (two
 // popcounts of windows per neighbour and word, before: one launch of 1,024
 // replicas x 10^5 steps at N = 64 took 559 cycles a step).
 //
