@@ -98,6 +98,7 @@ template <int NWMAX, int WPS>
 __global__ void __launch_bounds__(256, WPS == 2 || NWMAX > 6 ? 1 : 2) batch_kernel(const BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PairLink links[WPS == 2 ? 4 : 1];  // one per pair of an 8-warp CTA
+    static_assert(WPS == 1 || sizeof links == kPairLinkSmem, "shared memory of the links");
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     unsigned char* base = smem + static_cast<size_t>(warp) * a.smem_per_warp;
@@ -134,7 +135,7 @@ static const void* batch_fn(int nwmax, int wps) {
 cudaError_t batch_prepare(int nwmax, int wps, int warps_per_block, size_t smem_per_warp, int* max_blocks_per_sm) {
     const void* fn = batch_fn(nwmax, wps);
     const size_t smem = smem_per_warp * warps_per_block;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = allow_cta_smem(fn, wps, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(max_blocks_per_sm, fn, warps_per_block * 32, smem);
 }

@@ -14,8 +14,19 @@ namespace lgpu {
 // ints each) and the spins (96 nw bytes); see tabu_search.
 constexpr size_t tabu_scratch_bytes(int nw) { return 608u * static_cast<size_t>(nw); }
 
-// Shared memory of one CTA.
+// Shared memory of one CTA, and the part of it that the kernels on warp pairs declare (their links).
 constexpr size_t kCtaSmem = 227u * 1024u;
+constexpr size_t kPairLinkSmem = 128;
+
+// Lets a CTA of fn (wps warps per replica) take `smem` bytes of dynamic shared
+// memory.  The limit belongs to the function on its device, not to a launch, so
+// it is only ever raised to all there is: threads that set it to what their own
+// launch takes lower it between another thread's call and that thread's launch.
+inline cudaError_t allow_cta_smem(const void* fn, int wps, size_t smem) {
+    const size_t most = kCtaSmem - (wps == 2 ? kPairLinkSmem : 0);
+    if (smem > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
 
 // A mapping or a server with wpb warps per CTA is accepted while wpb warps of
 // `pop` population bytes and 256 nw bytes fit a CTA.  The search's scratch is
@@ -23,7 +34,7 @@ constexpr size_t kCtaSmem = 227u * 1024u;
 // quarter), which no result depends on.  `least`: warps that belong together.
 inline int cta_warps(int wpb, int least, size_t pop, int nw) {
     const auto padded = [](size_t b) { return (b + 15) & ~size_t{15}; };
-    const size_t links = least == 2 ? 128 : 0;  // static shared memory of the kernels on warp pairs
+    const size_t links = least == 2 ? kPairLinkSmem : 0;
     if (padded(pop + 256u * static_cast<size_t>(nw)) * wpb + links > kCtaSmem) return wpb;  // refused by the caller
     while (wpb > least && padded(pop + tabu_scratch_bytes(nw)) * wpb + links > kCtaSmem) wpb /= 2;
     return wpb;
@@ -125,7 +136,9 @@ cudaError_t launch_skew(const uint64_t* d_seqs, int N, int64_t B, int32_t* d_out
 int serve_class_nw(int N);
 size_t serve_smem_per_warp(int nw, int K);
 // Resident CTAs per SM of the class-nw quantum kernel with wps warps per slot
-// (occupancy API); pairs exist for even nw only (serve_pairs_supported).
+// (occupancy API); pairs exist for even nw only (serve_pairs_supported).  Comes
+// before the first launch of that kernel on a device: it raises the limit that
+// the launch's shared memory may need (allow_cta_smem).
 int serve_pairs_supported(int nw);
 cudaError_t serve_blocks_per_sm(int nw, int wps, int warps_per_block, size_t smem_per_warp, int* blocks);
 // One quantum of the slots of one word-count class, wps warps per slot (an

@@ -213,13 +213,15 @@ __global__ void __launch_bounds__(32, kMinBlocks) tabu_kernel(const TabuArgs a) 
     }
 }
 
+// The largest population and scratch of one warp fit the dynamic shared memory
+// that every launch may take, so the launches below set no limit of their kernels
+// (see allow_cta_smem).
+static_assert(LABS_MAX_K * (2 * LABS_MAX_W + 1) * 4 + tabu_scratch_bytes(2 * LABS_MAX_W) + 15 <= 48 * 1024,
+              "a warp's shared memory");
+
 template <int NW, bool TRACE, bool SKEW, int BLOCKS>
 cudaError_t launch_mts_b(const MtsArgs& a, cudaStream_t stream) {
-    const size_t smem = a.smem_per_warp;
-    cudaError_t e = cudaFuncSetAttribute(mts_kernel<NW, TRACE, SKEW, BLOCKS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    mts_kernel<NW, TRACE, SKEW, BLOCKS><<<warp_grid(a.replicas), 32, smem, stream>>>(a);
+    mts_kernel<NW, TRACE, SKEW, BLOCKS><<<warp_grid(a.replicas), 32, a.smem_per_warp, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -256,11 +258,7 @@ cudaError_t launch_mts_family(const MtsArgs& a, cudaStream_t stream) {
 
 template <int NW, bool SKEW, int BLOCKS>
 cudaError_t launch_resume_b(const ResumeArgs& a, cudaStream_t stream) {
-    const size_t smem = a.m.smem_per_warp;
-    cudaError_t e = cudaFuncSetAttribute(mts_resume_kernel<NW, SKEW, BLOCKS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    mts_resume_kernel<NW, SKEW, BLOCKS><<<warp_grid(a.m.replicas), 32, smem, stream>>>(a);
+    mts_resume_kernel<NW, SKEW, BLOCKS><<<warp_grid(a.m.replicas), 32, a.m.smem_per_warp, stream>>>(a);
     return cudaGetLastError();
 }
 

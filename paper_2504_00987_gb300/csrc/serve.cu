@@ -135,6 +135,7 @@ template <int NW, int WPS>
 __global__ void __launch_bounds__(256, WPS == 2 || NW > 6 ? 1 : 2) serve_quantum_kernel(const ServeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PairLink links[WPS == 2 ? 4 : 1];  // one per pair of an 8-warp CTA
+    static_assert(WPS == 1 || sizeof links == kPairLinkSmem, "shared memory of the links");
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     PairLink* link = WPS == 2 ? &links[warp >> 1] : nullptr;
@@ -187,7 +188,7 @@ int serve_pairs_supported(int nw) { return nw % 2 == 0 ? 1 : 0; }
 cudaError_t serve_blocks_per_sm(int nw, int wps, int warps_per_block, size_t smem_per_warp, int* blocks) {
     const void* fn = serve_fn(nw, wps);
     const size_t smem = smem_per_warp * warps_per_block;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = allow_cta_smem(fn, wps, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, warps_per_block * 32, smem);
 }
@@ -198,16 +199,13 @@ cudaError_t launch_serve_quantum(const ServeArgs& a, int nw, int wps, int warps_
     const size_t smem = a.smem_per_warp * warps_per_block;
     const int slots_per_block = warps_per_block / wps;
     const int blocks = (a.n_active + slots_per_block - 1) / slots_per_block;
-    const void* fn = serve_fn(nw, wps);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(blocks));
     cfg.blockDim = dim3(static_cast<unsigned>(warps_per_block * 32));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     void* args[] = {const_cast<ServeArgs*>(&a)};
-    return cudaLaunchKernelExC(&cfg, fn, args);
+    return cudaLaunchKernelExC(&cfg, serve_fn(nw, wps), args);
 }
 
 }  // namespace lgpu
