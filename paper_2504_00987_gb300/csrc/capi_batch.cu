@@ -84,21 +84,12 @@ size_t smem_of(const labs_instance* h, int64_t n) {
     return s;
 }
 
-// Warps per CTA that a mapping's wpb becomes for these instances (cta_warps
-// of the largest population, whose footprint every warp of the launch gets).
+// Warps per CTA that a mapping's wpb becomes for these instances; 0: it does not fit.
 int cta_warps_of(const labs_instance* h, int64_t n, int wpb, int wps) {
-    const labs_instance* top = nullptr;
-    size_t most = 0;
-    for (int64_t i = 0; i < n; ++i) {
-        const size_t b = lgpu::mts_smem_per_warp(h[i].N, h[i].K);
-        if (b > most) {
-            most = b;
-            top = h + i;
-        }
-    }
-    if (top == nullptr) return wpb;
-    const int nw = 2 * ((top->N + 63) / 64);
-    return lgpu::cta_warps(wpb, wps, static_cast<size_t>(top->K) * (nw + 1) * 4, nw);
+    size_t asked = 0;
+    for (int64_t i = 0; i < n; ++i)
+        asked = std::max(asked, lgpu::warp_smem_asked(2 * ((h[i].N + 63) / 64), h[i].K));
+    return lgpu::cta_warps(wpb, wps, asked, smem_of(h, n));
 }
 
 std::vector<int32_t> queue_order(const labs_instance* h, int64_t n, int order) {
@@ -239,6 +230,7 @@ int32_t labs_autotune(const labs_instance* h_inst, int64_t n, labs_stream_t stre
             if (wpb < wps) continue;
             int maxb = 0;
             const int cta = cta_warps_of(h_inst, n, wpb, wps);
+            if (e == cudaSuccess && cta == 0) e = cudaErrorInvalidValue;
             if (e == cudaSuccess) e = lgpu::batch_prepare(nwmax, wps, cta, spw, &maxb);
             if (e != cudaSuccess) break;
             maxb /= wpb / cta;  // CTAs of wpb warps
@@ -305,12 +297,13 @@ int32_t labs_batch_create(const labs_instance* h_inst, int64_t n, const labs_map
     b->d_queue = d.queue;
     int maxb = 0;
     const int cta = cta_warps_of(h_inst, n, m.warps_per_block, wps_of(m));
+    if (e == cudaSuccess && cta == 0) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) e = lgpu::batch_prepare(b->nwmax, wps_of(m), cta, b->smem_per_warp, &maxb);
     if (e == cudaSuccess && maxb < 1) {
         labs_batch_destroy(b);
         return fail(LABS_EINVAL, "mapping does not fit on an SM (warps_per_block=%d)", m.warps_per_block);
     }
-    b->blocks = sm_count() * std::min(m.blocks_per_sm * (m.warps_per_block / cta), std::max(maxb, 1));
+    if (e == cudaSuccess) b->blocks = sm_count() * std::min(m.blocks_per_sm * (m.warps_per_block / cta), maxb);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {

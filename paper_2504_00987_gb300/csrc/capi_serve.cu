@@ -464,15 +464,25 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
         return nullptr;
     }
     const int top = class_of(o->max_N);
-    const size_t pop_max = static_cast<size_t>(o->max_K) * (kClassNw[top] + 1) * 4;
-    const int cta = lgpu::cta_warps(o->warps_per_block, 1, pop_max, kClassNw[top]);
-    if (lgpu::serve_smem_per_warp(kClassNw[top], o->max_K) * cta > lgpu::kCtaSmem) {
+    const int cta = lgpu::cta_warps(o->warps_per_block, 1, lgpu::warp_smem_asked(kClassNw[top], o->max_K),
+                                    lgpu::serve_smem_per_warp(kClassNw[top], o->max_K));
+    if (cta == 0) {
         fail(LABS_EINVAL, "max_N/max_K populations of one block exceed shared memory");
         return nullptr;
     }
     if (o->warps_per_request < 0 || o->warps_per_request > 2) {
         fail(LABS_EINVAL, "warps_per_request must be 0, 1 or 2");
         return nullptr;
+    }
+    int pair_wpb = 2;
+    if (o->warps_per_request == 2) {  // the largest even word count sets the pairs' CTA
+        const int nw = kClassNw[top] % 2 == 0 ? kClassNw[top] : kClassNw[top - 1];
+        pair_wpb = lgpu::cta_warps(std::max(2, o->warps_per_block), 2, lgpu::warp_smem_asked(nw, o->max_K),
+                                   lgpu::serve_smem_per_warp(nw, o->max_K));
+        if (pair_wpb == 0) {
+            fail(LABS_EINVAL, "max_N/max_K populations of one block of warp pairs exceed shared memory");
+            return nullptr;
+        }
     }
     if (o->quantum_steps < 1 || o->queue_capacity < 0 || o->hbm_budget_bytes < 0 ||
         o->quantum_timeout_ms < 0 || o->quantum_us < 0 || o->quantum_us > (int64_t{1} << 40)) {
@@ -487,7 +497,7 @@ labs_server* labs_serve_create(const labs_serve_opts* o) {
     s->opts = *o;
     s->opts.warps_per_block = cta;
     s->sms = sm_count();
-    s->pair_wpb = std::max(2, cta);
+    s->pair_wpb = pair_wpb;
     cudaGetDevice(&s->device);
     // the arena: hbm_budget_bytes, or room for max_slots requests of (max_N, max_K)
     labs_request biggest{};

@@ -28,15 +28,23 @@ inline cudaError_t allow_cta_smem(const void* fn, int wps, size_t smem) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
 }
 
-// A mapping or a server with wpb warps per CTA is accepted while wpb warps of
-// `pop` population bytes and 256 nw bytes fit a CTA.  The search's scratch is
-// larger: where wpb warps do not fit with it, the CTA runs half as many (or a
-// quarter), which no result depends on.  `least`: warps that belong together.
-inline int cta_warps(int wpb, int least, size_t pop, int nw) {
-    const auto padded = [](size_t b) { return (b + 15) & ~size_t{15}; };
-    const size_t links = least == 2 ? kPairLinkSmem : 0;
-    if (padded(pop + 256u * static_cast<size_t>(nw)) * wpb + links > kCtaSmem) return wpb;  // refused by the caller
-    while (wpb > least && padded(pop + tabu_scratch_bytes(nw)) * wpb + links > kCtaSmem) wpb /= 2;
+// Shared memory by which a warp's request is judged: K sequences of nw words,
+// their energies and 256 nw bytes.
+inline size_t warp_smem_asked(int nw, int K) {
+    const size_t b = static_cast<size_t>(K) * (nw + 1) * 4 + 256u * static_cast<size_t>(nw);
+    return (b + 15) & ~size_t{15};
+}
+
+// Warps that a CTA asked to have wpb warps runs; 0 if that is refused.  A mapping
+// or a server is accepted while wpb warps of `asked` bytes fit a CTA, `asked` the
+// largest warp_smem_asked of what it may run.  A warp takes `need` bytes, which is
+// more (the search's scratch): where wpb of those do not fit, the CTA runs half as
+// many (or a quarter), which no result depends on.  `least`: warps that belong
+// together, 2 for the kernels on warp pairs.
+inline int cta_warps(int wpb, int least, size_t asked, size_t need) {
+    const size_t most = kCtaSmem - (least == 2 ? kPairLinkSmem : 0);
+    if (asked * wpb > most) return 0;
+    while (wpb > least && need * wpb > most) wpb /= 2;
     return wpb;
 }
 
