@@ -51,7 +51,9 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_thread_kernel(const uin
 }
 
 // A warp takes ROWS consecutive sequences at a time, so that one's loads and
-// reduction overlap the others' work.
+// reduction overlap the others' work.  ROWS = 1: each warp has one sequence, and
+// the kernel no loop, whose bounds took a fifth of a small call (E and C, 4,000
+// sequences of N = 64 2.15 / 1.67 us with / without it).
 template <int NW, int ROWS>
 __global__ void __launch_bounds__(kEnergyThreads) energy_warp_kernel(const uint32_t* __restrict__ seqs, int N,
                                                                      int64_t B, int32_t* __restrict__ E,
@@ -62,12 +64,12 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_warp_kernel(const uint3
     uint32_t mask[NW];
     pair_masks<NW, false>(N, lane, mask);
     for (int64_t b0 = warp * ROWS; b0 < B; b0 += warps * ROWS) {
-        const int rows = static_cast<int>(min(static_cast<int64_t>(ROWS), B - b0));
+        const int rows = ROWS == 1 ? 1 : static_cast<int>(min(static_cast<int64_t>(ROWS), B - b0));
         int32_t sq[ROWS];
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             uint32_t s[NW];
-            load_row<NW>(seqs, min(b0 + r, B - 1), N, s);
+            load_row<NW>(seqs, ROWS == 1 ? b0 : min(b0 + r, B - 1), N, s);
             int32_t c[NW];
             lane_correlations<NW>(s, mask, N, lane, c);
             sq[r] = lane >= 1 ? c[0] * c[0] : 0;  // C_0 does not count
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_warp_kernel(const uint3
             e = lane == r ? t : e;
         }
         if (lane < rows) E[b0 + lane] = e;
+        if constexpr (ROWS == 1) break;
     }
 }
 
@@ -95,8 +98,8 @@ template <int NW, int ROWS>
 static void launch_energy_warps(const uint32_t* seqs, int N, int64_t B, int32_t* d_E, int32_t* d_C,
                                 cudaStream_t stream) {
     constexpr int per_block = kEnergyThreads / 32 * ROWS;
-    const int64_t wave = static_cast<int64_t>(lcapi::sm_count()) * 8;  // 64 warps on every SM
-    const int64_t blocks = std::min((B + per_block - 1) / per_block, wave);
+    int64_t blocks = (B + per_block - 1) / per_block;
+    if (ROWS > 1) blocks = std::min(blocks, static_cast<int64_t>(lcapi::sm_count()) * 8);  // 64 warps on every SM
     energy_warp_kernel<NW, ROWS><<<static_cast<unsigned>(blocks), kEnergyThreads, 0, stream>>>(seqs, N, B, d_E, d_C);
 }
 
@@ -104,9 +107,11 @@ static void launch_energy_warps(const uint32_t* seqs, int N, int64_t B, int32_t*
 // thread's chain grows with NW^2, and below that it outlasts the warps'
 // (us, warps / threads: N = 64 1.8 / 2.4 at B = 4,000, 3.0 / 2.5 at 20,000;
 // N = 120 2.9 / 3.8 at 10,000, 5.5 / 5.9 at 40,000, 24 / 18 at 300,000;
-// N = 256 12 / 17 at 40,000, 25 / 24 at 100,000).  A warp
-// takes one sequence at a time up to 32 per SM, four from there (E and C at
-// N = 120: 2.0 / 2.5 at 1,000, 5.5 / 4.4 at 20,000).
+// N = 256 12 / 17 at 40,000, 25 / 24 at 100,000).  A warp takes one sequence
+// up to 48 per SM, at seven and eight words up to 192, and four at a time from
+// there (E and C, one / four: N = 64 1.94 / 2.05 at B = 6,000, 2.17 / 2.06 at
+// 9,728; N = 128 2.35 / 2.60 and 2.89 / 2.69; N = 256 3.57 / 4.62 at 6,000,
+// 8.1 / 8.7 at 20,000, 11.4 / 11.6 at 30,000, 21.0 / 20.0 at 60,000).
 template <int NW>
 static cudaError_t launch_energy_w(const uint64_t* d_seqs, int N, int64_t B, int32_t* d_E,
                                    int32_t* d_C, cudaStream_t stream) {
@@ -115,7 +120,7 @@ static cudaError_t launch_energy_w(const uint64_t* d_seqs, int N, int64_t B, int
     if (d_C == nullptr && B > sms * 8 * NW * NW) {
         const int64_t blocks = (B + kEnergyThreads - 1) / kEnergyThreads;
         energy_thread_kernel<NW><<<static_cast<unsigned>(blocks), kEnergyThreads, 0, stream>>>(seqs, N, B, d_E);
-    } else if (B <= sms * 32) {
+    } else if (B <= sms * (NW >= 7 ? 192 : 48)) {
         launch_energy_warps<NW, 1>(seqs, N, B, d_E, d_C, stream);
     } else {
         launch_energy_warps<NW, 4>(seqs, N, B, d_E, d_C, stream);

@@ -68,3 +68,23 @@ def test_energies_and_correlations(labs, orc, N):
             E, C = labs.energy_batch(d, N, with_C=True)
             assert np.array_equal(E.cpu().numpy(), want)
             assert np.array_equal(C.cpu().numpy(), np.tile(C0, (rep, 1))[:B])
+
+
+@pytest.mark.parametrize("N", [3, 31, 64, 65, 128, 161, 192, 193, 224, 225, 256])
+def test_energies_on_either_side_of_four_rows_a_warp(labs, orc, N):
+    """The largest batch of one sequence a warp and the smallest of four, E with and
+    without C; the rows past the first few repeat them, so the oracle is asked once."""
+    few = 37
+    a = sequences(N, few, dirty=True)
+    ora = [orc.energy(x, N, with_C=True) for x in sequences(N, few, dirty=False)]
+    E0 = np.array([e for e, _ in ora], dtype=np.int32)
+    C0 = np.array([c for _, c in ora], dtype=np.int32)
+    line = (192 if N > 192 else 48) * torch.cuda.get_device_properties(0).multi_processor_count
+    for B in (line, line + 1, line + 3):
+        rep = -(-B // few)
+        d = dev(np.tile(a, (rep, 1))[:B])
+        want = np.tile(E0, rep)[:B]
+        E, C = labs.energy_batch(d, N, with_C=True)
+        assert np.array_equal(E.cpu().numpy(), want)
+        assert np.array_equal(C.cpu().numpy(), np.tile(C0, (rep, 1))[:B])
+        assert np.array_equal(labs.energy_batch(d, N).cpu().numpy(), want)
