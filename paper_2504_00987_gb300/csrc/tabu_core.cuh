@@ -20,6 +20,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "kernels.h"
 #include "labs_device.cuh"
 
 namespace lgpu {
@@ -172,10 +173,10 @@ __device__ __forceinline__ bool pair_exchange(PairLink* link, int half, uint32_t
     return ok;
 }
 
-// Scratch of one warp's tabu search (ints): V (2 NB), C (2 NB), spins (3 NB
-// bytes), NB = 32 NW; a multiple of 16 bytes.
+// Scratch of one warp's tabu search (ints): what the launches leave room for
+// (tabu_scratch_bytes).
 template <int NW>
-constexpr int kTabuScratchInts = 128 * NW + 24 * NW;
+constexpr int kTabuScratchInts = static_cast<int>(tabu_scratch_bytes(NW) / sizeof(int32_t));
 
 // V_m = sum_a x_a x_{m-a} for m = lane + 32i <= N - 1, stored at V[m] (or at
 // V[2N - 2 - m], MIRROR, where X is the sequence reversed): bits X and their
@@ -208,6 +209,9 @@ __device__ __forceinline__ uint2 step_draws(uint2 key, uint32_t inst, uint32_t g
 // at S[i], i = -NB .. 2 NB - 1.
 template <int NW>
 struct TabuScratch {
+    static_assert(4 * (2 * 32 * NW) + 4 * (2 * 32 * NW) + 3 * 32 * NW == tabu_scratch_bytes(NW) &&
+                      tabu_scratch_bytes(NW) % 16 == 0,
+                  "V, C and the spins take the scratch");
     int32_t* V;
     int32_t* C;
     int8_t* S;
