@@ -80,3 +80,13 @@ def test_traffic_record_matches_the_kernel(bench):
     rec = json.load(open(bench.TRAFFIC_FILE))
     assert rec["kernel_hash"] == bench.kernel_hash()
     assert 0 < rec["bytes_per_launch"] < 1 << 20
+
+
+def test_roofline_counts_what_a_step_does(bench):
+    """Seven operations a move and step over the issue rate: a fraction of a pipe, so
+    below one at any length and any time the kernel can reach."""
+    r = bench.roofline(64, 1024 * 100_000, 15.06)
+    assert r["achieved"] == pytest.approx(7 * 64 * 1024 * 100_000 / 15.06e-3 / 1e9)
+    assert r["peak"] == pytest.approx(152 * 128 * 2.07) and r["frac"] == pytest.approx(r["achieved"] / r["peak"])
+    assert 0.07 < r["frac"] < 0.08 and r["traffic"] is None
+    assert bench.roofline(256, 1216 * 20_000, 8.11, 100)["frac"] < 1.0
