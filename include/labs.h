@@ -188,7 +188,7 @@ typedef struct labs_instance {
     uint64_t instance;
 } labs_instance;
 
-#define LABS_ORDER_LPT 0   /* queue longest instance first (pair-term budget) */
+#define LABS_ORDER_LPT 0   /* queue the largest pair-term budget, N (N - 1) a step, first */
 #define LABS_ORDER_GIVEN 1 /* queue in the given order */
 
 /* How a batch is mapped on the GPU. */

@@ -3,10 +3,10 @@
 // CTAs of warps_per_block warps on every SM); each replica unit (one warp,
 // or with warps_per_seq = 2 a pair of warps that split every step's
 // neighbours) takes the next instance from a device-wide queue (one
-// atomicAdd per instance, ordered longest first by the host), runs it to
-// its stop condition with the replica engine and writes its result at the
-// instance's original index.  Instances of different word counts share the
-// launch: the unit dispatches on W = ceil(N/64) per instance.  Per-instance
+// atomicAdd per instance, ordered by the host, largest pair-term budget first),
+// runs it to its stop condition with the replica engine and writes its result at
+// the instance's original index.  Instances of different word counts share the
+// launch: the unit runs 2 ceil(N/64) words, chosen per instance.  Per-instance
 // results do not depend on the mapping or on the other instances (every
 // draw is keyed by the instance's own seed and instance number).
 #include <cuda_runtime.h>
@@ -79,9 +79,12 @@ __device__ __forceinline__ void batch_unit(const BatchArgs& a, unsigned char* ba
         if (W == 1) {
             run_instance<2, WPS, HALF>(cfg, base, out, lane, link, &xseq);
         } else if (W == 2) {
-            // four words up to N = 128: a three-word path in this kernel cost the
-            // four-word one its registers (172 -> 128) and the batch's makespan,
-            // which the longest (largest-N) instances set, 12 % on GB300
+            // Even word counts only.  Paths of three and five words as well, at the
+            // same 128 registers, took 1.63 against 1.88 ms for 64 instances of
+            // N = 65..96 x 10,000 steps, 2.18 against 3.50 for N = 129..160, 2.58
+            // against 2.56 for N = 193..256, and 27.0 against 27.7 for 512 of
+            // N = 40..127 x 10 N^2 steps (one warp each, one GB300); they are not
+            // compiled in.
             if constexpr (NWMAX >= 4) run_instance<4, WPS, HALF>(cfg, base, out, lane, link, &xseq);
         } else if (W == 3) {
             if constexpr (NWMAX >= 6) run_instance<6, WPS, HALF>(cfg, base, out, lane, link, &xseq);

@@ -4,14 +4,16 @@
 //  - E only, many sequences: one thread per sequence (NW words in registers).
 //  - E and C, or few sequences: one warp per sequence, lane l computes C_k for
 //    k = l + 32q, so each row of C is written by consecutive lanes
-//    (coalesced); the masks of a lane are those of every sequence, so a warp
-//    keeps them and takes one sequence after the other.
+//    (coalesced); the masks of a lane are those of every sequence, so a warp of
+//    a large batch keeps them and takes one group of sequences after the other.
 // What bounds them: popcounts, 8 cycles of the XU pipe a warp and 8 of them per
 // 32 values of k at N = 120 after the full adders (10 words), 51 us for 10^6
-// sequences; with C, the stores of its rows (16-byte stores through shared
-// memory took 35 us where these take 33).  On GB300, N = 120: 10^6 energies
-// 56 us (masks rebuilt for every word and round, no adders: 151), 300,000 with
-// C 33 us, 4.3 TB/s (57); 100 energies 2.0 us on the device (8.8).
+// sequences; with C, instructions (82 a warp and sequence at N = 127, issued in
+// 65 % of the cycles, the ALU pipe as full) and too few warps to cover the rows'
+// loads, not the rows' stores (a fill of as many bytes takes 22.6 us of its 34.8;
+// 16-byte stores through shared memory took 35 us where these take 33).  On
+// GB300, N = 120: 10^6 energies 57 us (masks rebuilt for every word and round, no
+// adders: 151), 300,000 with C 33 us (57); 100 energies 1.5 us on the device (8.6).
 #include <cuda_runtime.h>
 
 #include <algorithm>

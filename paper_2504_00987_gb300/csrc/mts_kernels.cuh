@@ -2,8 +2,9 @@
 // tabu search (Algorithm 2 / Algorithm 4) kernels, templated on the word
 // count, tracing and the skew-symmetric restriction (Sec. II.C).  One warp
 // runs one replica: its population lives in the warp's slice of shared
-// memory (K packed sequences and their energies), its pivot, correlations
-// and tabu list in registers.  Replicas never synchronise with each other;
+// memory (K packed sequences and their energies), followed by its tabu search's
+// correlations, self-convolution and spins; the neighbours' keys and the tabu
+// list are in registers.  Replicas never synchronise with each other;
 // the only cross-replica state is the optional global termination flag.
 // mts.cu instantiates the unrestricted kernels, mts_skew.cu the restricted
 // ones and mts_resume.cu the resumable ones (both kinds), so each
@@ -23,15 +24,21 @@ namespace lgpu {
 // search of N = 201 takes 73 us on an SM of its own and 87 us beside three
 // others; 5,000 of them, of uneven length, 331 us instead of 394).
 // Sixteen CTAs per SM leave 128 registers a thread.  Without a bound the
-// compiler aims at more warps than the workloads put on an SM and squeezes
-// the step (N = 64 64 registers, 217 cycles a step for a lone warp against
-// 204; N = 120 96, 359 against 330).
+// compiler aims at more warps than the workloads put on an SM and squeezes the
+// short steps, and it takes too many registers for sixteen at six words (cycles
+// a step, without / with the bound, one warp alone on a sub-partition and four:
+// N = 64 199 / 190 and 502 / 497, N = 92 294 / 297 and 658 / 650, N = 120 411 /
+// 331 and 795 / 751, N = 160 363 / 366 and 870 / 868, N = 192 419 / 434 and
+// 1,142 / 1,027).
 constexpr int kMinBlocks = 16;
 // Seven and eight words take up to 255 registers while at most eight replicas
 // fall on an SM, which is all those leave room for (128 / 255 registers, one
 // GB300: 152 replicas of N = 256 x 20,000 steps 5.95 / 5.12 ms, 608 of N = 200
 // 5.85 / 4.69, 1,216 of N = 256 8.11 / 7.41); with more, 16 warps on an SM win
-// (a step of 2,432 at N = 256: 1,356 / 1,429 cycles).
+// (a step of 2,432 at N = 256: 1,356 / 1,429 cycles).  Fewer words gain little or
+// lose (cycles a step, 128 / 255 registers, a lone warp: N = 192 434 / 426, N = 160
+// 366 / 398, N = 120 331 / 334), and so do searches (100 of N = 201 70.5 / 71.8 us,
+// 5,000 307 / 322; of N = 256 98 / 93 and 435 / 437): those keep 128.
 constexpr int kFewBlocks = 8;
 template <int NW>
 inline bool few_replicas(int64_t n) {
@@ -232,13 +239,14 @@ cudaError_t launch_mts_t(const MtsArgs& a, cudaStream_t stream) {
     return launch_mts_b<NW, TRACE, SKEW, kMinBlocks>(a, stream);
 }
 
-// 32-bit words per sequence in registers.  A step's work grows with them, so
-// every count has its kernel (one word against two, one N = 24 instance of
-// 2,000 generations: 5.72 ms against 6.60; seven against eight, 5,000 searches
-// at N = 201: 309 us against 343).
+// 32-bit words per sequence in registers, for launches and searches.  A step's
+// work grows with them, so every count has its kernel (one word against two, one
+// N = 24 instance of 2,000 generations: 5.72 ms against 6.60; seven against
+// eight, 5,000 searches at N = 201: 309 us against 343).
 inline int word_count(int N) { return (N + 31) / 32; }
 
-// Words per member of a resumable record: part of the record's layout.
+// Words per member of a resumable record, and of the kernels that read it: part
+// of the record's layout, so N <= 32 runs two words there and N = 193..224 eight.
 inline int record_words(int N) { return N <= 64 ? 2 : N <= 96 ? 3 : N <= 128 ? 4 : N <= 160 ? 5 : N <= 192 ? 6 : 8; }
 
 template <bool SKEW>

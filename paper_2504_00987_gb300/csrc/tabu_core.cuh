@@ -377,10 +377,13 @@ __device__ TabuOut tabu_search(uint32_t (&seq)[NW], const int N, const uint2 key
     static_assert(WPS == 1 || (WPS == 2 && NW % 2 == 0 && HALF >= 0 && HALF < 2), "warps per sequence");
     constexpr int QB = HALF * (NW / WPS), QE = (HALF + 1) * (NW / WPS);  // this warp's q
     // A drawn tie is scored by a second copy of the scoring code at three and
-    // four words, and through the loop of the first at two, where that copy is
-    // as long as the rest of the step, and from five words on, where it costs
-    // registers (cycles a step, one warp alone, with / without the copy: N = 64
-    // 243 / 217, N = 120 343 / 355, N = 160 375 / 358, N = 256 502 / 475).
+    // four words, and through the loop of the first at the others, where the copy
+    // costs registers (cycles a step, with / without the copy, one warp alone on
+    // a sub-partition and four: N = 64 231 / 190 and 525 / 497, N = 92 297 / 273
+    // and 650 / 608, N = 120 331 / 311 and 751 / 756, N = 160 367 / 366 and 868 /
+    // 867, N = 256 503 / 487 and 1,369 / 1,356).  The line was drawn when the copy
+    // was ahead at N = 120 (343 / 355); as the step is now it only pays there with
+    // four warps on a sub-partition, and at three words not at all.
     constexpr bool kRecompute = NW <= 4 && NW > 2;
     constexpr int32_t kLow = 511;  // key bits below the energy change
     constexpr int32_t kNone = INT_MAX & ~kLow;  // no candidate: above every key, low bits those of j = 0

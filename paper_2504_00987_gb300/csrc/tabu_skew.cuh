@@ -31,7 +31,7 @@
 //
 // What bounds it: like tabu_search, the serial chain of a step, here with two
 // dependent updates in it.  Two warps on a sub-partition, N = 101, 1,216
-// replicas x 10^4 steps: 4.41 ms on GB300 (scoring every step from the bit
+// replicas x 10^4 steps: 3.73 ms on GB300 (scoring every step from the bit
 // planes of C_k: 17.28 ms).
 #pragma once
 
